@@ -14,6 +14,8 @@
 // cell has non-negative components, then ordered by decreasing |n_k|.
 #include <math.h>
 
+#include <algorithm>
+
 #include "fsl_internal.cuh"
 #include "mlp_common.cuh"
 
@@ -97,9 +99,8 @@ __device__ __forceinline__ double uniform_at(unsigned long long seed, unsigned l
     return (double)(splitmix64_at(seed, k) >> 11) * (1.0 / 9007199254740992.0);
 }
 
-// mean curvature at the point of the ellipsoid sum (y/a)^2 = 1 (body frame)
-// nearest to o (body frame): x_k = a_k^2 o_k / (a_k^2 + t), bisection on t
-__device__ double nearest_mean_curvature(const double a[3], const double o[3]) {
+// the multiplier t of the nearest surface point by bisection (see below)
+__device__ __noinline__ double nearest_bisect(const double a[3], const double o[3]) {
     double lo = -fmin(a[0] * a[0], fmin(a[1] * a[1], a[2] * a[2])) * (1.0 - 1e-15);
     double hi = fmax(1.0, fmax(fabs(o[0]), fmax(fabs(o[1]), fabs(o[2]))) * fmax(a[0], fmax(a[1], a[2])));
     auto gfun = [&](double t) {
@@ -116,7 +117,31 @@ __device__ double nearest_mean_curvature(const double a[3], const double o[3]) {
         if (gfun(mid) > 0.0) lo = mid;
         else hi = mid;
     }
-    const double t = 0.5 * (lo + hi);
+    return 0.5 * (lo + hi);
+}
+
+// mean curvature at the point of the ellipsoid sum (y/a)^2 = 1 (body frame)
+// nearest to o (body frame): x_k = a_k^2 o_k / (a_k^2 + t)
+__device__ double nearest_mean_curvature(const double a[3], const double o[3]) {
+    // |q(t)| = 1 with q_k = a_k o_k / (a_k^2 + t): Newton's method on 1/|q|, which
+    // is nearly linear in t, from the left of the largest root, where no single
+    // |q_k| exceeds 1; it converges in four or five steps.  Points it does not
+    // settle for (the ellipsoid's centre and focal set) take the bisection.
+    double t = -1e300;
+    for (int k = 0; k < 3; ++k) t = fmax(t, fabs(a[k] * o[k]) - a[k] * a[k]);
+    bool done = false;
+    for (int it = 0; it < 12 && !done; ++it) {
+        double q2 = 0.0, dq = 0.0;
+        for (int k = 0; k < 3; ++k) {
+            const double r = 1.0 / (a[k] * a[k] + t), q = a[k] * o[k] * r;
+            q2 += q * q;
+            dq += q * q * r;
+        }
+        const double st = q2 / dq * (sqrt(q2) - 1.0);
+        done = fabs(st) <= 4e-16 * fmax(fabs(t), a[0] * a[0]);
+        t += st;
+    }
+    if (!done || !(t > -fmin(a[0] * a[0], fmin(a[1] * a[1], a[2] * a[2])) * (1.0 - 1e-15))) t = nearest_bisect(a, o);
     double gr[3], hs[3], gn2 = 0.0, trh = 0.0, ghg = 0.0;
     for (int k = 0; k < 3; ++k) {
         const double x = a[k] * a[k] * o[k] / (a[k] * a[k] + t);
@@ -130,70 +155,210 @@ __device__ double nearest_mean_curvature(const double a[3], const double o[3]) {
     return (gn2 * trh - ghg) / (2.0 * gn2 * gn);
 }
 
-// one block per stencil: thread e < 125 samples cell e
-__global__ void __launch_bounds__(128) k_mlp_stencils(int n, const float *axes, const float *quat, const float *dir,
-                                                      const float *delta, const int *invert, int sub, float noise,
-                                                      unsigned long long noise_seed, __nv_bfloat16 *X, float *target) {
-    __shared__ float Rm[9], C[3], ax[3];
-    __shared__ float st[125];
-    __shared__ Canon cs;
-    for (long long k = blockIdx.x; k < n; k += gridDim.x) {
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            const double w = quat[4 * k], x = quat[4 * k + 1], y = quat[4 * k + 2], z = quat[4 * k + 3];
-            const double R[9] = {1 - 2 * (y * y + z * z), 2 * (x * y - w * z), 2 * (x * z + w * y),
-                                 2 * (x * y + w * z), 1 - 2 * (x * x + z * z), 2 * (y * z - w * x),
-                                 2 * (x * z - w * y), 2 * (y * z + w * x), 1 - 2 * (x * x + y * y)};
-            const double a[3] = {axes[3 * k], axes[3 * k + 1], axes[3 * k + 2]};
-            const double d[3] = {dir[3 * k], dir[3 * k + 1], dir[3 * k + 2]};
-            const double sc = 1.0 / sqrt((d[0] / a[0]) * (d[0] / a[0]) + (d[1] / a[1]) * (d[1] / a[1]) +
-                                         (d[2] / a[2]) * (d[2] / a[2]));
-            double c[3], o[3];
+// rotation (row-major, FP64) and centre of stencil k's ellipsoid, its surface
+// point at `delta` from the middle cell's centre
+__device__ __forceinline__ void stencil_frame(long long k, const float *axes, const float *quat, const float *dir,
+                                              const float *delta, double R[9], double a[3], double c[3]) {
+    const double w = quat[4 * k], x = quat[4 * k + 1], y = quat[4 * k + 2], z = quat[4 * k + 3];
+    const double M[9] = {1 - 2 * (y * y + z * z), 2 * (x * y - w * z), 2 * (x * z + w * y),
+                         2 * (x * y + w * z), 1 - 2 * (x * x + z * z), 2 * (y * z - w * x),
+                         2 * (x * z - w * y), 2 * (y * z + w * x), 1 - 2 * (x * x + y * y)};
+    for (int e = 0; e < 9; ++e) R[e] = M[e];
+    for (int r = 0; r < 3; ++r) a[r] = axes[3 * k + r];
+    const double d[3] = {dir[3 * k], dir[3 * k + 1], dir[3 * k + 2]};
+    const double sc = 1.0 / sqrt((d[0] / a[0]) * (d[0] / a[0]) + (d[1] / a[1]) * (d[1] / a[1]) +
+                                 (d[2] / a[2]) * (d[2] / a[2]));
+    for (int r = 0; r < 3; ++r) c[r] = delta[3 * k + r] - (R[3 * r] * d[0] + R[3 * r + 1] * d[1] + R[3 * r + 2] * d[2]) * sc;
+}
+
+// Targets, one thread per stencil: the FP64 rate (2 FMA per clock and SM) bounds
+// them, so every lane of a warp has a stencil of its own.
+__global__ void __launch_bounds__(128) k_mlp_targets(int n, const float *axes, const float *quat, const float *dir,
+                                                     const float *delta, const int *invert, float *target) {
+    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
+        double R[9], a[3], c[3], o[3];
+        stencil_frame(k, axes, quat, dir, delta, R, a, c);
+        for (int r = 0; r < 3; ++r) o[r] = -(R[r] * c[0] + R[3 + r] * c[1] + R[6 + r] * c[2]);  // R^T (0 - C)
+        const double H = nearest_mean_curvature(a, o);
+        target[k] = (float)(invert[k] ? -H : H);
+    }
+}
+
+// Stencils, one warp for `per` consecutive ones.  Lane l < per sets up stencil
+// l (FP64), then the warp takes them one at a time:
+//   cells    the lanes decide the cells the surface |A^-1 R^T (p - C)| = 1 cannot
+//            cut, from the value and gradient at the cell's centre; about 45 of
+//            125 stay open
+//   columns  the same for the sub x sub columns of samples of the open cells
+//            (a quarter stays open), queued so that the 32 lanes always sample
+//            32 open columns
+//   noise    on the partially filled cells, packed onto the lanes (FP64)
+// and the canonical BF16 row leaves in one 8-byte store per lane.  One block of
+// 125 sampling threads per stencil, one of which also bisected for the target
+// in FP64, took 16 ms for 65536 stencils at sub = 8; this takes 1.55 ms and the
+// targets 0.08.
+constexpr int ST_WARPS = 4;
+
+struct StWarp {
+    float frame[32][16];  // R (9), C (3), semi-axes (3), least semi-axis
+    float st[128];
+    int cnt[128];
+    int queue[64];
+    uint8_t open[128];
+    __nv_bfloat16 row[128];
+};
+
+__global__ void __launch_bounds__(32 * ST_WARPS) k_mlp_stencils(int n, int per, const float *axes, const float *quat,
+                                                                const float *dir, const float *delta,
+                                                                const int *invert, int sub, float noise,
+                                                                unsigned long long noise_seed, __nv_bfloat16 *X) {
+    __shared__ StWarp smem[ST_WARPS];
+    StWarp &s = smem[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+    const unsigned full = 0xffffffffu;
+    const long long groups = ((long long)n + per - 1) / per, nw = (long long)gridDim.x * ST_WARPS;
+    const int S2 = sub * sub, tot = S2 * sub;
+    const int magic = (65536 + sub - 1) / sub;  // c / sub = (c magic) >> 16 for c < 1024, sub <= 32
+    const float h = 1.0f / sub, half = 0.5f * (float)(sub - 1) * h + 1e-6f;  // half a column of samples
+    for (long long g = (long long)blockIdx.x * ST_WARPS + (threadIdx.x >> 5); g < groups; g += nw) {
+        const int m = (int)min((long long)per, n - g * per);
+        if (lane < m) {
+            double R[9], a[3], c[3];
+            stencil_frame(g * per + lane, axes, quat, dir, delta, R, a, c);
+            float *f = s.frame[lane];
+            for (int e = 0; e < 9; ++e) f[e] = (float)R[e];
             for (int r = 0; r < 3; ++r) {
-                c[r] = delta[3 * k + r] - (R[3 * r] * d[0] + R[3 * r + 1] * d[1] + R[3 * r + 2] * d[2]) * sc;
-                C[r] = (float)c[r];
-                ax[r] = (float)a[r];
+                f[9 + r] = (float)c[r];
+                f[12 + r] = (float)a[r];
             }
-            for (int e = 0; e < 9; ++e) Rm[e] = (float)R[e];
-            for (int r = 0; r < 3; ++r) o[r] = -(R[r] * c[0] + R[3 + r] * c[1] + R[6 + r] * c[2]);  // R^T (0 - C)
-            const double H = nearest_mean_curvature(a, o);
-            target[k] = (float)(invert[k] ? -H : H);
+            f[15] = fminf(f[12], fminf(f[13], f[14]));
         }
-        __syncthreads();
-        const int e = threadIdx.x;
-        if (e < 125) {
-            const int i = e / 25 - 2, j = (e / 5) % 5 - 2, l = e % 5 - 2;
-            const float inv_a0 = 1.0f / ax[0], inv_a1 = 1.0f / ax[1], inv_a2 = 1.0f / ax[2];
-            const float h = 1.0f / sub;
-            int cnt = 0;
-            for (int sx = 0; sx < sub; ++sx) {
-                const float px = i + (sx + 0.5f) * h - 0.5f - C[0];
-                for (int sy = 0; sy < sub; ++sy) {
-                    const float py = j + (sy + 0.5f) * h - 0.5f - C[1];
-                    for (int sz = 0; sz < sub; ++sz) {
-                        const float pz = l + (sz + 0.5f) * h - 0.5f - C[2];
-                        const float y0 = (Rm[0] * px + Rm[3] * py + Rm[6] * pz) * inv_a0;
-                        const float y1 = (Rm[1] * px + Rm[4] * py + Rm[7] * pz) * inv_a1;
-                        const float y2 = (Rm[2] * px + Rm[5] * py + Rm[8] * pz) * inv_a2;
-                        cnt += (y0 * y0 + y1 * y1 + y2 * y2 <= 1.0f) ? 1 : 0;
-                    }
+        __syncwarp();
+        for (int q = 0; q < m; ++q) {
+            const long long k = g * per + q;
+            const float *f = s.frame[q];
+            float Rm[9], C[3];
+#pragma unroll
+            for (int e = 0; e < 9; ++e) Rm[e] = f[e];
+#pragma unroll
+            for (int r = 0; r < 3; ++r) C[r] = f[9 + r];
+            const float inv_a0 = 1.0f / f[12], inv_a1 = 1.0f / f[13], inv_a2 = 1.0f / f[14], lip = 1.0f / f[15];
+            // r = |A^-1 R^T (p - C)| is a norm of p - C: over a displacement v its change is
+            // at most |grad r . v| + (lip |v|)^2 / (2 (r - lip |v|)), and at most lip |v|.
+            // reach = |v|, gz = bound of |grad r . v| / |v|.  1: all within the reach
+            // inside, 0: none, -1: open.  tol is far above the rounding of the sample test.
+            const float tol = 4e-6f * ((fabsf(C[0]) + fabsf(C[1]) + fabsf(C[2]) + 8.0f) * lip + 1.0f);
+            auto decide = [&](float px, float py, float pz, float reach, bool along_z) {
+                const float y0 = (Rm[0] * px + Rm[3] * py + Rm[6] * pz) * inv_a0;
+                const float y1 = (Rm[1] * px + Rm[4] * py + Rm[7] * pz) * inv_a1;
+                const float y2 = (Rm[2] * px + Rm[5] * py + Rm[8] * pz) * inv_a2;
+                const float r2 = fmaxf(y0 * y0 + y1 * y1 + y2 * y2, 1e-30f), ir = rsqrtf(r2), r = r2 * ir;
+                const float v0 = y0 * inv_a0, v1 = y1 * inv_a1, v2 = y2 * inv_a2;
+                const float gr = along_z ? fabsf(Rm[6] * v0 + Rm[7] * v1 + Rm[8] * v2) * ir
+                                         : sqrtf(v0 * v0 + v1 * v1 + v2 * v2) * ir;
+                const float lr = lip * reach, rest = r - lr;
+                float b = lr;
+                if (rest > 0.1f) b = fminf(b, 1.0001f * gr * reach + __fdividef(0.5001f * lr * lr, rest));
+                b += tol * (1.0f + r);
+                return 1.0f - r > b ? 1 : (r - 1.0f > b ? 0 : -1);
+            };
+            int nopen = 0;
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const int e = lane + 32 * t;
+                int v = 0;
+                if (e < 125)
+                    v = decide((float)(e / 25 - 2) - C[0], (float)((e / 5) % 5 - 2) - C[1], (float)(e % 5 - 2) - C[2], 0.8661f,
+                               false);
+                s.cnt[e] = v == 1 ? tot : 0;
+                const unsigned mk = __ballot_sync(full, v < 0);
+                if (v < 0) s.open[nopen + __popc(mk & ((1u << lane) - 1u))] = (uint8_t)e;
+                nopen += __popc(mk);
+            }
+            __syncwarp();
+            // one column of samples: cell e, column (sx, sy)
+            auto column = [&](int item) {
+                const int slot = item >> 10, col = item & 1023;
+                const int e = s.open[slot], sx = (col * magic) >> 16, sy = col - sx * sub;
+                const int i = e / 25 - 2, j = (e / 5) % 5 - 2, l = e % 5 - 2;
+                const float px = i + (sx + 0.5f) * h - 0.5f - C[0], py = j + (sy + 0.5f) * h - 0.5f - C[1];
+                const float b0 = fmaf(Rm[3], py, __fmul_rn(Rm[0], px)), b1 = fmaf(Rm[4], py, __fmul_rn(Rm[1], px)),
+                            b2 = fmaf(Rm[5], py, __fmul_rn(Rm[2], px));
+                int cnt = 0;
+#pragma unroll 4
+                for (int sz = 0; sz < sub; ++sz) {
+                    const float pz = l + (sz + 0.5f) * h - 0.5f - C[2];
+                    const float y0 = fmaf(Rm[6], pz, b0) * inv_a0, y1 = fmaf(Rm[7], pz, b1) * inv_a1,
+                                y2 = fmaf(Rm[8], pz, b2) * inv_a2;
+                    cnt += (y0 * y0 + y1 * y1 + y2 * y2 <= 1.0f) ? 1 : 0;
                 }
+                if (cnt) atomicAdd(&s.cnt[e], cnt);
+            };
+            int queued = 0, slot = 0, col = lane;
+            for (int base = 0; base < nopen * S2; base += 32) {  // warp-uniform
+                while (col >= S2) {
+                    col -= S2;
+                    ++slot;
+                }
+                int v = 0;
+                if (slot < nopen) {
+                    const int e = s.open[slot], sx = (col * magic) >> 16, sy = col - sx * sub;
+                    v = decide((float)(e / 25 - 2) + (sx + 0.5f) * h - 0.5f - C[0],
+                               (float)((e / 5) % 5 - 2) + (sy + 0.5f) * h - 0.5f - C[1], (float)(e % 5 - 2) - C[2], half, true);
+                    if (v == 1) atomicAdd(&s.cnt[e], sub);
+                }
+                const unsigned mk = __ballot_sync(full, v < 0);
+                if (v < 0) s.queue[queued + __popc(mk & ((1u << lane) - 1u))] = (slot << 10) | col;
+                queued += __popc(mk);
+                __syncwarp();
+                if (queued >= 32) {
+                    queued -= 32;
+                    column(s.queue[queued + lane]);
+                    __syncwarp();
+                }
+                col += 32;
             }
-            const int tot = sub * sub * sub;
-            float phi = (float)(invert[k] ? tot - cnt : cnt) / (float)tot;
-            if (noise > 0.f && phi > 0.f && phi < 1.f) {
-                const unsigned long long idx = (unsigned long long)k * 125ULL + e;
-                const double u1 = uniform_at(noise_seed, 2 * idx), u2 = uniform_at(noise_seed, 2 * idx + 1);
-                const float nrm = (float)(sqrt(-2.0 * log1p(-u1)) * cos(6.283185307179586 * u2));
-                phi = fminf(fmaxf(phi + noise * nrm, 0.f), 1.f);
+            if (lane < queued) column(s.queue[lane]);
+            __syncwarp();
+            // fill levels; the partially filled cells (all among the open ones) take the noise
+            const bool inv = invert[k] != 0;
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const int e = lane + 32 * t;
+                s.st[e] = (float)(inv ? tot - s.cnt[e] : s.cnt[e]) / (float)tot;
             }
-            st[e] = phi;
+            __syncwarp();
+            if (noise > 0.f) {
+                int np = 0;
+                for (int b = 0; b < nopen; b += 32) {
+                    const int e = b + lane < nopen ? s.open[b + lane] : 0;
+                    const bool part = b + lane < nopen && s.st[e] > 0.f && s.st[e] < 1.f;
+                    const unsigned mk = __ballot_sync(full, part);
+                    __syncwarp();
+                    if (part) s.open[np + __popc(mk & ((1u << lane) - 1u))] = (uint8_t)e;
+                    np += __popc(mk);
+                    __syncwarp();
+                }
+                for (int b = lane; b < np; b += 32) {
+                    const int e = s.open[b];
+                    const unsigned long long idx = (unsigned long long)k * 125ULL + e;
+                    const double u1 = uniform_at(noise_seed, 2 * idx), u2 = uniform_at(noise_seed, 2 * idx + 1);
+                    // 1 - u1 is exact (u1 is a multiple of 2^-53)
+                    const float nrm = (float)(sqrt(-2.0 * log(1.0 - u1)) * cospi(2.0 * u2));
+                    s.st[e] = fminf(fmaxf(s.st[e] + noise * nrm, 0.f), 1.f);
+                }
+                __syncwarp();
+            }
+            const Canon cs = canon_of(s.st);
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const int e = lane + 32 * t;
+                s.row[e < 125 ? canon_index(cs, e) : e] = __float2bfloat16_rn(e < 125 ? 2.0f * s.st[e] - 1.0f : 0.f);
+            }
+            __syncwarp();
+            reinterpret_cast<uint2 *>(X + k * MK)[lane] = reinterpret_cast<const uint2 *>(s.row)[lane];
+            __syncwarp();
         }
-        __syncthreads();
-        if (threadIdx.x == 0) cs = canon_of(st);
-        __syncthreads();
-        if (e < 125) X[k * MK + canon_index(cs, e)] = __float2bfloat16_rn(2.0f * st[e] - 1.0f);
-        else X[k * MK + e] = __float2bfloat16_rn(0.f);
     }
 }
 
@@ -238,9 +403,15 @@ int fsl_mlp_stencils(int n, const float *axes, const float *quat, const float *d
     if (n < 0 || !axes || !quat || !dir || !delta || !invert || !X || !target || sub < 1 || sub > 32 || noise < 0.f)
         return FSL_EINVAL;
     if (n == 0) return FSL_OK;
-    const int grid = n < 65536 ? n : 65536;
-    k_mlp_stencils<<<grid, 128, 0, (cudaStream_t)stream>>>(n, axes, quat, dir, delta, invert, sub, noise, noise_seed,
-                                                          static_cast<__nv_bfloat16 *>(X), target);
+    cudaStream_t s = (cudaStream_t)stream;
+    const int wide = 152 * 16 * ST_WARPS;  // warps of a full GPU
+    // a few stencils per warp fill the lanes of the FP64 set-up; fewer where that would leave SMs idle
+    const int per = std::min(8, std::max(1, n / wide));
+    const long long groups = ((long long)n + per - 1) / per;
+    const int grid = (int)std::min<long long>((groups + ST_WARPS - 1) / ST_WARPS, 152 * 64);
+    k_mlp_targets<<<std::min((n + 127) / 128, 152 * 16), 128, 0, s>>>(n, axes, quat, dir, delta, invert, target);
+    k_mlp_stencils<<<grid, 32 * ST_WARPS, 0, s>>>(n, per, axes, quat, dir, delta, invert, sub, noise, noise_seed,
+                                                 static_cast<__nv_bfloat16 *>(X));
     return cudaGetLastError() == cudaSuccess ? FSL_OK : FSL_ECUDA;
 }
 
