@@ -106,6 +106,9 @@ Dev make_dev(const fsl_params &p, const fsl_fields &f) {
     d.ny = p.ny;
     d.nz = p.nz;
     d.N = (long long)p.nx * p.ny * p.nz;
+    d.by_nx = fast_div(p.nx);
+    d.by_ny = fast_div(p.ny);
+    d.by_nsegx = fast_div((p.nx + SEG - 1) / SEG);
     d.mass = f.mass;
     d.phi = f.phi;
     d.kappa = f.kappa;

@@ -95,9 +95,27 @@ inline cudaError_t launch_pdl(void (*kernel)(P...), int grid, int block, cudaStr
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// Division of 0 <= n < 2^31 by a divisor fixed at set-up: floor(n m / 2^(31+k))
+// with 2^k >= divisor and m = ceil(2^(31+k) / divisor) is exact, and takes two
+// instructions instead of the twenty of a division by a variable.
+struct FastDiv {
+    uint32_t m;
+    int shift;
+};
+inline FastDiv fast_div(int divisor) {
+    int k = 0;
+    while ((1ll << k) < divisor) ++k;
+    const unsigned long long p = 1ull << (31 + k);
+    return FastDiv{(uint32_t)((p + (unsigned)divisor - 1) / (unsigned)divisor), 31 + k};
+}
+__host__ __device__ __forceinline__ int div_by(int n, const FastDiv &f) {
+    return (int)(((unsigned long long)(unsigned)n * f.m) >> f.shift);
+}
+
 // kernel argument block (passed by value)
 struct Dev {
     int nx, ny, nz;
+    FastDiv by_nx, by_ny, by_nsegx;
     long long N;
     const void *fsrc;  // post-collision PDFs at t
     void *fdst;        // post-collision PDFs at t+1
@@ -191,7 +209,7 @@ template <>
 struct Store<FSL_F32> {
     using T = float;
     __device__ static __forceinline__ float ld(const void *p, long long k, int q, const Dev &) {
-        return __ldg(static_cast<const float *>(p) + k);
+        return static_cast<const float *>(p)[k];
     }
     __device__ static __forceinline__ float ldcg(const void *p, long long k, int q, const Dev &) {
         return __ldcg(static_cast<const float *>(p) + k);
@@ -199,12 +217,19 @@ struct Store<FSL_F32> {
     __device__ static __forceinline__ void st(void *p, long long k, int q, float v, const Dev &) {
         static_cast<float *>(p)[k] = v;
     }
+    // direction q of cell i
+    __device__ static __forceinline__ float ld_at(const void *p, int q, unsigned i, const Dev &d) {
+        return (static_cast<const float *>(p) + (long long)q * d.N)[i];
+    }
+    __device__ static __forceinline__ void st_at(void *p, int q, unsigned i, float v, const Dev &d) {
+        (static_cast<float *>(p) + (long long)q * d.N)[i] = v;
+    }
 };
 template <>
 struct Store<FSL_F16_OFS> {
     using T = __half;
     __device__ static __forceinline__ float ld(const void *p, long long k, int q, const Dev &d) {
-        return fmaf(__half2float(__ldg(static_cast<const __half *>(p) + k)), d.inv_scale, wq(q));
+        return fmaf(__half2float(static_cast<const __half *>(p)[k]), d.inv_scale, wq(q));
     }
     __device__ static __forceinline__ float ldcg(const void *p, long long k, int q, const Dev &d) {
         return fmaf(__half2float(__ldcg(static_cast<const __half *>(p) + k)), d.inv_scale, wq(q));
@@ -212,18 +237,32 @@ struct Store<FSL_F16_OFS> {
     __device__ static __forceinline__ void st(void *p, long long k, int q, float v, const Dev &d) {
         static_cast<__half *>(p)[k] = __float2half_rn((v - wq(q)) * d.scale);
     }
+    __device__ static __forceinline__ float ld_at(const void *p, int q, unsigned i, const Dev &d) {
+        const __half h = (static_cast<const __half *>(p) + (long long)q * d.N)[i];
+        return fmaf(__half2float(h), d.inv_scale, wq(q));
+    }
+    __device__ static __forceinline__ void st_at(void *p, int q, unsigned i, float v, const Dev &d) {
+        (static_cast<__half *>(p) + (long long)q * d.N)[i] = __float2half_rn((v - wq(q)) * d.scale);
+    }
 };
 template <>
 struct Store<FSL_BF16_OFS> {
     using T = __nv_bfloat16;
     __device__ static __forceinline__ float ld(const void *p, long long k, int q, const Dev &d) {
-        return fmaf(__bfloat162float(__ldg(static_cast<const __nv_bfloat16 *>(p) + k)), d.inv_scale, wq(q));
+        return fmaf(__bfloat162float(static_cast<const __nv_bfloat16 *>(p)[k]), d.inv_scale, wq(q));
     }
     __device__ static __forceinline__ float ldcg(const void *p, long long k, int q, const Dev &d) {
         return fmaf(__bfloat162float(__ldcg(static_cast<const __nv_bfloat16 *>(p) + k)), d.inv_scale, wq(q));
     }
     __device__ static __forceinline__ void st(void *p, long long k, int q, float v, const Dev &d) {
         static_cast<__nv_bfloat16 *>(p)[k] = __float2bfloat16_rn((v - wq(q)) * d.scale);
+    }
+    __device__ static __forceinline__ float ld_at(const void *p, int q, unsigned i, const Dev &d) {
+        const __nv_bfloat16 h = (static_cast<const __nv_bfloat16 *>(p) + (long long)q * d.N)[i];
+        return fmaf(__bfloat162float(h), d.inv_scale, wq(q));
+    }
+    __device__ static __forceinline__ void st_at(void *p, int q, unsigned i, float v, const Dev &d) {
+        (static_cast<__nv_bfloat16 *>(p) + (long long)q * d.N)[i] = __float2bfloat16_rn((v - wq(q)) * d.scale);
     }
 };
 
@@ -239,9 +278,9 @@ __device__ __forceinline__ int nbr_index(const Dev &d, int x, int y, int z, int 
 }
 
 __device__ __forceinline__ void cell_coords(const Dev &d, int i, int &x, int &y, int &z) {
-    const int row = i / d.nx;
+    const int row = div_by(i, d.by_nx);
     x = i - row * d.nx;
-    z = row / d.ny;
+    z = div_by(row, d.by_ny);
     y = row - z * d.ny;
 }
 
@@ -305,7 +344,7 @@ __device__ __forceinline__ void warp_uniform_loop(int n, Body body) {
 }
 
 __device__ __forceinline__ int seg_of(const Dev &d, int i) {
-    const int row = i / d.nx;
+    const int row = div_by(i, d.by_nx);
     return (i - row * d.nx) / SEG + d.nsegx * row;
 }
 

@@ -11,17 +11,11 @@
 //              level with wetting normals at obstacle cells (Sec. II.A).
 //   k_tr       triangle-fan curvature of the PLIC points (Sec. II.B).
 // The per-cell arithmetic is in curv_common.cuh.
-#include "curv_common.cuh"
+#include "step_common.cuh"
 
 namespace fslk {
 
 constexpr int LIST_THREADS = 128;
-
-// Parker-Youngs normal of a cell next to an obstacle (reflected fill levels at
-// the obstacle cells); out of line, so that the loop of k_normals stays short
-__device__ __noinline__ void normal_near_wall(const Dev &d, int x, int y, int z, float nv[3]) {
-    parker_youngs<float>([&](int dx, int dy, int dz) { return phi_ext(d, x + dx, y + dy, z + dz); }, nv);
-}
 
 // The first kernel of a step also runs the step prologue (counters, bubble
 // pressure); every later kernel of the step is ordered after it on the stream.
@@ -31,24 +25,8 @@ __global__ void __launch_bounds__(LIST_THREADS) k_normals(Dev d) {
     block_counts<1>(d.counts, {d.cif}, cnt);
     const int n = cnt[0];
     if (blockIdx.x == 0 && threadIdx.x == 0) step_prologue(d);
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-        const int i = d.iflist[k];
-        int x, y, z;
-        cell_coords(d, i, x, y, z);
-        // the 27 fill levels are loaded with the cell's type (one round); a cell
-        // next to a wall takes the reflected ones instead, out of line
-        float ph[27];
-#pragma unroll
-        for (int t = 0; t < 27; ++t) ph[t] = d.phi[nbr_index(d, x, y, z, t % 3 - 1, (t / 3) % 3 - 1, t / 9 - 1)];
-        const uint8_t fl = d.flags[i];
-        float nv[3], a;
-        if (fl & B_NEAR)
-            normal_near_wall(d, x, y, z, nv);
-        else
-            parker_youngs<float>([&](int dx, int dy, int dz) { return ph[(dz + 1) * 9 + (dy + 1) * 3 + (dx + 1)]; }, nv);
-        const bool ok = unit_normal_offset<float>(nv, ph[13], d.plic_iters, a);
-        d.normal[i] = ok ? make_float4(nv[0], nv[1], nv[2], a) : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x)
+        normal_cell(d, d.iflist[k]);
 }
 
 __global__ void __launch_bounds__(LIST_THREADS) k_lsqr_fast(Dev d, float *kappa_out) {
