@@ -81,11 +81,11 @@ __device__ __forceinline__ void pdl_enter() {
 }
 
 template <typename... P, typename... A>
-inline cudaError_t launch_pdl(void (*kernel)(P...), int grid, int block, cudaStream_t s, A... args) {
+inline cudaError_t launch_pdl_smem(void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t s, A... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -93,6 +93,10 @@ inline cudaError_t launch_pdl(void (*kernel)(P...), int grid, int block, cudaStr
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+template <typename... P, typename... A>
+inline cudaError_t launch_pdl(void (*kernel)(P...), int grid, int block, cudaStream_t s, A... args) {
+    return launch_pdl_smem(kernel, grid, block, 0, s, args...);
 }
 
 // Division of 0 <= n < 2^31 by a divisor fixed at set-up: floor(n m / 2^(31+k))
@@ -377,10 +381,11 @@ int launch_mlp_forward_tc(const uint8_t *params, const __nv_bfloat16 *X, int n, 
 int mlp_tc_status(bool reset);
 // one training step's forward, deltas and gradient partials on the tensor cores,
 // one CTA per 128 rows of the batch (rows perm[row0 ..] of X, or row0 .. when
-// perm is null); part holds mlp_tile_partial_floats(n) floats, lpart one double per tile
+// perm is null); follows: the kernel before it on the stream is the update of the
+// step before, so X, target and perm may be read while that one still runs; part holds mlp_tile_partial_floats(n) floats, lpart one double per tile
 size_t mlp_tile_partial_floats(int n);
 int launch_mlp_train_tile(const uint8_t *params, const __nv_bfloat16 *X, const float *target, const int64_t *perm,
-                          long long row0, int n, long long n_all, float *part, double *lpart, cudaStream_t s);
+                          long long row0, int n, long long n_all, bool follows, float *part, double *lpart, cudaStream_t s);
 void launch_fin_frozen(const Dev &d, cudaStream_t s);
 // bubble model: liquid cells, non-obstacle cells and the fixed-point fill-level
 // sum of the current state into d.bub_i (entries of the current parity and [4])

@@ -44,16 +44,21 @@ __global__ void __launch_bounds__(256) k_mlp_tile_reduce(const float *part, cons
                                                          uint8_t *params, float *master, float *m, float *v, float lr,
                                                          float bc1, float bc2) {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e == 0 && loss) {
+    pdl_enter();
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x < 32 && loss) {  // in the last block, which is half idle
         double l = 0.0;
-        for (int t = 0; t < ntiles; ++t) l += lpart[t];
-        loss[0] = (float)(l / n);
+        for (int t = threadIdx.x; t < ntiles; t += 32) l += lpart[t];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+        if (threadIdx.x == 0) loss[0] = (float)(l / n);
     }
     if (e >= M_COUNT) return;
+    // 16 partials in flight: the sum is a chain of adds, the loads need not be
     float acc = 0.f;
     if (e < M_W3) {
         const int mat = e / (MK * MK), k = e % (MK * MK);
         const float *P = part + (size_t)mat * MK * MK + k;
+#pragma unroll 16
         for (int t = 0; t < ntiles; ++t) acc += P[(size_t)t * PART_STRIDE];
     } else {
         int vec, c = 0;
@@ -62,6 +67,7 @@ __global__ void __launch_bounds__(256) k_mlp_tile_reduce(const float *part, cons
         else if (e < M_B3) { vec = 1; c = e - M_B2; }
         else { vec = 3; }
         const float *P = part + (size_t)2 * MK * MK + (size_t)vec * MK + c;
+#pragma unroll 16
         for (int t = 0; t < ntiles; ++t) acc += P[(size_t)t * PART_STRIDE];
     }
     if (grad) grad[e] = acc;
@@ -428,18 +434,18 @@ int fsl_mlp_status(int reset) { return mlp_tc_status(reset != 0); }
 // tile kernel over the batch rows perm[row0 .. row0 + n) of X (rows row0 ..
 // when perm is null), then the fixed-order reduction of its partials.
 static int mlp_step(const void *params, const void *X, const float *target, const int64_t *perm, long long row0, int n,
-                    long long n_all, float *loss_dev, void *workspace, float *grad_out, void *params_rw, float *master,
-                    float *m, float *v, float lr, int step, cudaStream_t s) {
+                    long long n_all, bool follows, float *loss_dev, void *workspace, float *grad_out, void *params_rw,
+                    float *master, float *m, float *v, float lr, int step, cudaStream_t s) {
     char *ws = static_cast<char *>(workspace);
     const TrainWs L = train_ws(n);
     float *part = reinterpret_cast<float *>(ws + L.part);
     double *lpart = reinterpret_cast<double *>(ws + L.lpart);
     const int rc = launch_mlp_train_tile(static_cast<const uint8_t *>(params), static_cast<const __nv_bfloat16 *>(X),
-                                         target, perm, row0, n, n_all, part, lpart, s);
+                                         target, perm, row0, n, n_all, follows, part, lpart, s);
     if (rc != FSL_OK) return rc;
     const float bc1 = master ? (float)(1.0 - pow(0.9, step)) : 1.f, bc2 = master ? (float)(1.0 - pow(0.999, step)) : 1.f;
-    k_mlp_tile_reduce<<<(M_COUNT + 255) / 256, 256, 0, s>>>(part, lpart, (n + MK - 1) / MK, n, grad_out, loss_dev,
-                                                           static_cast<uint8_t *>(params_rw), master, m, v, lr, bc1, bc2);
+    launch_pdl(k_mlp_tile_reduce, (M_COUNT + 255) / 256, 256, s, (const float *)part, (const double *)lpart,
+               (n + MK - 1) / MK, n, grad_out, loss_dev, static_cast<uint8_t *>(params_rw), master, m, v, lr, bc1, bc2);
     return cudaGetLastError() == cudaSuccess ? FSL_OK : FSL_ECUDA;
 }
 
@@ -447,7 +453,7 @@ int fsl_mlp_gradients(const void *params, const void *X, const float *target, in
                       void *workspace, void *stream) {
     if (!params || !X || !target || !grad || !workspace || n <= 0) return FSL_EINVAL;
     if (reinterpret_cast<uintptr_t>(X) % 16 || reinterpret_cast<uintptr_t>(workspace) % 256) return FSL_EINVAL;
-    return mlp_step(params, X, target, nullptr, 0, n, n, loss_dev, workspace, grad, nullptr, nullptr, nullptr, nullptr,
+    return mlp_step(params, X, target, nullptr, 0, n, n, false, loss_dev, workspace, grad, nullptr, nullptr, nullptr, nullptr,
                     0.f, 1, (cudaStream_t)stream);
 }
 
@@ -456,7 +462,7 @@ int fsl_mlp_train_step(void *params, float *master, float *m, float *v, const vo
     if (!params || !master || !m || !v || !X || !target || !workspace || n <= 0 || step < 1 || !(lr > 0.f))
         return FSL_EINVAL;
     if (reinterpret_cast<uintptr_t>(X) % 16 || reinterpret_cast<uintptr_t>(workspace) % 256) return FSL_EINVAL;
-    return mlp_step(params, X, target, nullptr, 0, n, n, loss_dev, workspace, nullptr, params, master, m, v, lr, step,
+    return mlp_step(params, X, target, nullptr, 0, n, n, false, loss_dev, workspace, nullptr, params, master, m, v, lr, step,
                     (cudaStream_t)stream);
 }
 
@@ -477,7 +483,7 @@ int fsl_mlp_train_epoch(void *params, float *master, float *m, float *v, const v
     cudaStream_t s = (cudaStream_t)stream;
     const int nb = n / batch;
     for (int b = 0; b < nb; ++b) {
-        const int rc = mlp_step(params, X, target, perm, (long long)b * batch, batch, n,
+        const int rc = mlp_step(params, X, target, perm, (long long)b * batch, batch, n, b > 0,
                                 losses_dev ? losses_dev + b : nullptr, workspace, nullptr, params, master, m, v, lr,
                                 step0 + b + 1, s);
         if (rc != FSL_OK) return rc;

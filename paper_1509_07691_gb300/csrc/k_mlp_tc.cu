@@ -255,9 +255,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_mlp_forward_tc(const uint8_t 
 }
 
 // ---- the learned curvature inside the step, on the tensor cores -----------------
-// One CTA (16 warps) per SM, persistent over 128-cell tiles of the interface
-// list.  Warp w takes rows 8w .. 8w+7 of a tile: lane r < 8 finds cell r's
-// canonical order from its 3x3x3 fill levels, then the warp gathers the 5x5x5
+// One CTA (16 warps) per SM, persistent over tiles of up to 128 cells of the
+// interface list.  Warp w takes rows w, w + 16, ... of a tile: lane r < 8 finds
+// the canonical order from its 3x3x3 fill levels, then the warp gathers the 5x5x5
 // fill levels of four cells at a time straight into the canonical BF16 rows
 // of X (x = 2 phi - 1).  The two layers run as in k_mlp_forward_tc (MMAs into
 // TMEM, GELU epilogues; thread (row, column quarter) reads 32 accumulator
@@ -284,9 +284,6 @@ __global__ void __launch_bounds__(CV_THREADS, 1) k_mlp_curv_tc(Dev d, float *kap
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     CvSmem &s = *reinterpret_cast<CvSmem *>(smem_raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int cnt[1];
-    block_counts<1>(d.counts, {d.cif}, cnt);
-    const int n = cnt[0];
     const __nv_bfloat16 *wb = reinterpret_cast<const __nv_bfloat16 *>(d.mlp_params);
     const float *bias = reinterpret_cast<const float *>(d.mlp_params + MB_BIAS_TC);
     load_tile(reinterpret_cast<char *>(s.W1), wb, TILE, TILE);
@@ -310,6 +307,17 @@ __global__ void __launch_bounds__(CV_THREADS, 1) k_mlp_curv_tc(Dev d, float *kap
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    // the weights and the tensor memory are in place while the fit before this
+    // kernel still runs
+    pdl_enter();
+    int cnt[1];
+    block_counts<1>(d.counts, {d.cif}, cnt);
+    const int n = cnt[0];
+    // Rows per tile: the list in equal tiles over whole rounds of the CTAs.  In
+    // tiles of 128 a list of 59 k cells is 3.04 rounds of 152 CTAs, and the
+    // fourth costs as much as a full one.
+    const int span = gridDim.x * TILE, turns = (n + span - 1) / span;
+    const int trows = turns ? (n + gridDim.x * turns - 1) / (gridDim.x * turns) : 1;
     const uint32_t tmem = s.tmem_base;
     const int q4 = warp & 3, cq = warp >> 2;
     const uint32_t lane_base = (uint32_t)(32 * q4) << 16;  // this warp's TMEM lanes
@@ -319,45 +327,43 @@ __global__ void __launch_bounds__(CV_THREADS, 1) k_mlp_curv_tc(Dev d, float *kap
     char *Xb = reinterpret_cast<char *>(s.X);
     uint32_t phase = 0;
     int evaluated = 0, kept = 0;
-    for (long long t0 = (long long)blockIdx.x * TILE; t0 < n; t0 += (long long)gridDim.x * TILE) {
-        // ---- gather: rows r0 .. r0 + 7 of this warp
-        const int r0 = warp * 8;
+    for (long long t0 = (long long)blockIdx.x * trows; t0 < n; t0 += (long long)gridDim.x * trows) {
+        // ---- gather: rows warp, warp + 16, ... of this warp (tile rows past trows
+        // keep what they held: a row of the MMAs depends on its own row only)
+        const int m = (int)min((long long)trows, n - t0), mine = (m - warp + 15) >> 4;
         int cx0 = 0, cy0 = 0, cz0 = 0, ci = -1;
         CanonAffine ca{0, {0, 0, 0}};
-        if (lane < 8 && t0 + r0 + lane < n) {
-            ci = d.iflist[t0 + r0 + lane];
+        if (lane < mine) {
+            ci = d.iflist[t0 + warp + 16 * lane];
             cell_coords(d, ci, cx0, cy0, cz0);
             ca = canon_affine(
                 canon_at([&](int dx, int dy, int dz) { return d.phi[nbr_index(d, cx0, cy0, cz0, dx, dy, dz)]; }));
         }
-        if (lane < 8) s.cell[r0 + lane] = ci;
+        if (lane < 8) s.cell[warp + 16 * lane] = ci;
         unsigned obsm = 0u;
 #pragma unroll 4
-        for (int r = 0; r < 8; ++r) {
+        for (int r = 0; r < mine; ++r) {
             const int x = __shfl_sync(0xffffffffu, cx0, r), y = __shfl_sync(0xffffffffu, cy0, r),
                       z = __shfl_sync(0xffffffffu, cz0, r);
             const int cb = __shfl_sync(0xffffffffu, ca.base, r), s0 = __shfl_sync(0xffffffffu, ca.s[0], r),
                       s1 = __shfl_sync(0xffffffffu, ca.s[1], r), s2 = __shfl_sync(0xffffffffu, ca.s[2], r);
-            const bool rv = t0 + r0 + r < n;
+            const int row8 = warp + 16 * r;
 #pragma unroll
             for (int t = 0; t < 4; ++t) {
                 const int e = lane + 32 * t;
                 if (e < 125) {
-                    float v = 0.f;
-                    if (rv) {
-                        const int j = nbr_index(d, x, y, z, e / 25 - 2, (e / 5) % 5 - 2, e % 5 - 2);
-                        v = d.phi[j];
-                        obsm |= (d.flags[j] & T_OBS) ? (1u << r) : 0u;
-                    }
+                    const int j = nbr_index(d, x, y, z, e / 25 - 2, (e / 5) % 5 - 2, e % 5 - 2);
+                    const float v = d.phi[j];
+                    if (!d.inline_general) obsm |= (d.flags[j] & T_OBS) ? (1u << r) : 0u;  // no obstacles: no types to read
                     const int k = cb + (e / 25) * s0 + ((e / 5) % 5) * s1 + (e % 5) * s2;
-                    *reinterpret_cast<__nv_bfloat16 *>(Xb + tile_off(r0 + r, k)) = __float2bfloat16_rn(2.0f * v - 1.0f);
+                    *reinterpret_cast<__nv_bfloat16 *>(Xb + tile_off(row8, k)) = __float2bfloat16_rn(2.0f * v - 1.0f);
                 } else {
-                    *reinterpret_cast<__nv_bfloat16 *>(Xb + tile_off(r0 + r, e)) = __float2bfloat16_rn(0.f);
+                    *reinterpret_cast<__nv_bfloat16 *>(Xb + tile_off(row8, e)) = __float2bfloat16_rn(0.f);
                 }
             }
         }
         obsm = __reduce_or_sync(0xffffffffu, obsm);
-        if (lane < 8) s.wall[r0 + lane] = (obsm >> lane) & 1u;
+        if (lane < 8) s.wall[warp + 16 * lane] = (obsm >> lane) & 1u;
         proxy_fence();
         __syncthreads();
         // ---- layer 1
@@ -472,7 +478,7 @@ __device__ __forceinline__ float gelu_grad_tc(float x) {
 //   E4     the tile's partials to part[tile] (PART_STRIDE floats: dW1, dW2,
 //          then the column sums of d1, d2, d3 gelu(z2) and d3, that is db1,
 //          db2, dw3, db3 at [0]); the tile's loss terms (FP32 terms, FP64 sum
-//          in row order) to lpart[tile].
+//          in a fixed tree) to lpart[tile].
 // The operand layouts are those of the forward, delta and weight-gradient
 // kernels above (K-major tiles, transposes written element by element).  Column
 // sums reduce over the 32 rows of a warp by a fixed shuffle tree and over the
@@ -547,6 +553,25 @@ __global__ void __launch_bounds__(FT_THREADS, 1)
 #pragma unroll
         for (int e = 0; e < 8; ++e) *reinterpret_cast<__nv_bfloat16 *>(T4 + tile_off(k8 + e, r)) = e8[e];
     }
+    if (threadIdx.x < TILE) {
+        const int e = threadIdx.x;
+        const long long src = source(e);
+        s.valid[e] = src >= 0;
+        s.tgt[e] = src >= 0 ? target[src] : 0.f;
+    }
+    if (threadIdx.x == 0) {
+        mbar_init(&s.mbar, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s.tmem_base)),
+                     "r"(512)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    // the batch is staged while the update before it still runs; the weights are
+    // the first thing that depends on it
+    pdl_enter();
     load_tile(T1, wb, TILE, TILE);
     load_tile(T2, wb + TILE * TILE, TILE, TILE);
     for (int c = threadIdx.x; c < TILE * TILE / 8; c += blockDim.x) {  // T3[h][o] = W2[o][h]
@@ -561,21 +586,8 @@ __global__ void __launch_bounds__(FT_THREADS, 1)
         s.b1[e] = bias[e];
         s.b2[e] = bias[TILE + e];
         s.w3[e] = __bfloat162float(wb[2 * TILE * TILE + e]);
-        const long long src = source(e);
-        s.valid[e] = src >= 0;
-        s.tgt[e] = src >= 0 ? target[src] : 0.f;
     }
-    if (threadIdx.x == 0) {
-        s.b3 = bias[2 * TILE];
-        mbar_init(&s.mbar, 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s.tmem_base)),
-                     "r"(512)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
+    if (threadIdx.x == 0) s.b3 = bias[2 * TILE];
     proxy_fence();
     tc_fence_before();
     __syncthreads();
@@ -751,10 +763,11 @@ __global__ void __launch_bounds__(FT_THREADS, 1)
             for (int k = 0; k < 3; ++k) V[k * TILE + c] = ((s.colred[0][k][c] + s.colred[1][k][c]) + s.colred[2][k][c]) + s.colred[3][k][c];
             V[3 * TILE + c] = c == 0 ? ((s.colred[0][3][0] + s.colred[1][3][0]) + s.colred[2][3][0]) + s.colred[3][3][0] : 0.f;
         }
-        if (threadIdx.x == 0) {
-            double l = 0.0;
-            for (int r = 0; r < TILE; ++r) l += (double)s.lterm[r];
-            lpart[tile] = l;
+        if (warp == 15) {  // the tile's loss: four rows a lane, then a fixed tree (FP64)
+            double l = ((double)s.lterm[lane] + (double)s.lterm[lane + 32]) + ((double)s.lterm[lane + 64] + (double)s.lterm[lane + 96]);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+            if (lane == 0) lpart[tile] = l;
         }
     }
     tc_fence_before();
@@ -809,14 +822,15 @@ size_t mlp_tile_partial_floats(int n) { return (size_t)((n + TILE - 1) / TILE) *
 // one training-step tile kernel per 128 rows of the batch (one CTA per SM at
 // about 170 KB of shared memory and 512 TMEM columns)
 int launch_mlp_train_tile(const uint8_t *params, const __nv_bfloat16 *X, const float *target, const int64_t *perm,
-                          long long row0, int n, long long n_all, float *part, double *lpart, cudaStream_t s) {
+                          long long row0, int n, long long n_all, bool follows, float *part, double *lpart, cudaStream_t s) {
     int *st = status_ptr();
     if (!st) return FSL_ECUDA;
     const size_t sm = sizeof(FtSmem) + 1024;
     if (cudaFuncSetAttribute(k_mlp_train_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess)
         return FSL_ECUDA;
-    k_mlp_train_tile<<<(n + TILE - 1) / TILE, FT_THREADS, sm, s>>>(params, X, target, perm, row0, n, n_all, part, lpart,
-                                                                   st);
+    const int tiles = (n + TILE - 1) / TILE;
+    if (follows) launch_pdl_smem(k_mlp_train_tile, tiles, FT_THREADS, sm, s, params, X, target, perm, row0, n, n_all, part, lpart, st);
+    else k_mlp_train_tile<<<tiles, FT_THREADS, sm, s>>>(params, X, target, perm, row0, n, n_all, part, lpart, st);
     return cudaGetLastError() == cudaSuccess ? FSL_OK : FSL_ECUDA;
 }
 
@@ -833,7 +847,7 @@ int launch_mlp_curv_tc(const Dev &d, float *kappa_out, cudaStream_t s) {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    k_mlp_curv_tc<<<sms > 0 ? sms : 1, CV_THREADS, sm, s>>>(d, kappa_out, st);
+    launch_pdl_smem(k_mlp_curv_tc, sms > 0 ? sms : 1, CV_THREADS, sm, s, d, kappa_out, st);
     return cudaGetLastError() == cudaSuccess ? FSL_OK : FSL_ECUDA;
 }
 
