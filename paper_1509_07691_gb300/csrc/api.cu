@@ -451,12 +451,9 @@ int fsl_init(const fsl_params *params, const fsl_fields *fields, const float *ph
         launch_init_types(d, obs, fields->flags[1], s);
         Dev d0 = dev_for(c, 0);
         d0.fdst = fields->f[0];
-        launch_init_state(d0, fields->flags[1], s);
+        // every cell of both buffers holds a defined value (w_q) from here on
+        launch_init_state(d0, fields->f[1], fields->flags[1], obs != nullptr, s);
         launch_seg_compact(d0, s);
-        // the second buffer starts as a copy, so every cell of both buffers
-        // holds a defined value (w_q away from the fluid) from here on
-        const size_t fbytes = (size_t)Q * N * pdf_elem_bytes(c->p.storage);
-        if (cudaMemcpyAsync(fields->f[1], fields->f[0], fbytes, cudaMemcpyDeviceToDevice, s) != cudaSuccess) break;
         if (cudaGetLastError() != cudaSuccess) break;
         if (read_near(c) != FSL_OK) break;
         c->parity = 0;

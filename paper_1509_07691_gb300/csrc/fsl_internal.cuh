@@ -221,6 +221,8 @@ struct Store<FSL_F32> {
     __device__ static __forceinline__ void st(void *p, long long k, int q, float v, const Dev &) {
         static_cast<float *>(p)[k] = v;
     }
+    // the stored form of value v of a direction of weight w
+    __device__ static __forceinline__ void put(float &o, float v, float w, const Dev &) { o = v; }
     // direction q of cell i
     __device__ static __forceinline__ float ld_at(const void *p, int q, unsigned i, const Dev &d) {
         return (static_cast<const float *>(p) + (long long)q * d.N)[i];
@@ -241,6 +243,7 @@ struct Store<FSL_F16_OFS> {
     __device__ static __forceinline__ void st(void *p, long long k, int q, float v, const Dev &d) {
         static_cast<__half *>(p)[k] = __float2half_rn((v - wq(q)) * d.scale);
     }
+    __device__ static __forceinline__ void put(__half &o, float v, float w, const Dev &d) { o = __float2half_rn((v - w) * d.scale); }
     __device__ static __forceinline__ float ld_at(const void *p, int q, unsigned i, const Dev &d) {
         const __half h = (static_cast<const __half *>(p) + (long long)q * d.N)[i];
         return fmaf(__half2float(h), d.inv_scale, wq(q));
@@ -261,6 +264,7 @@ struct Store<FSL_BF16_OFS> {
     __device__ static __forceinline__ void st(void *p, long long k, int q, float v, const Dev &d) {
         static_cast<__nv_bfloat16 *>(p)[k] = __float2bfloat16_rn((v - wq(q)) * d.scale);
     }
+    __device__ static __forceinline__ void put(__nv_bfloat16 &o, float v, float w, const Dev &d) { o = __float2bfloat16_rn((v - w) * d.scale); }
     __device__ static __forceinline__ float ld_at(const void *p, int q, unsigned i, const Dev &d) {
         const __nv_bfloat16 h = (static_cast<const __nv_bfloat16 *>(p) + (long long)q * d.N)[i];
         return fmaf(__bfloat162float(h), d.inv_scale, wq(q));
@@ -355,7 +359,9 @@ __device__ __forceinline__ int seg_of(const Dev &d, int i) {
 // ---- launch wrappers (defined in the .cu files) -------------------------------
 void launch_fill_geometry(const fsl_params &p, const fsl_geometry &g, float *phi, cudaStream_t s);
 void launch_init_types(const Dev &d, const uint8_t *obstacle, uint8_t *tmp, cudaStream_t s);
-void launch_init_state(const Dev &d, const uint8_t *tmp, cudaStream_t s);
+// w_q into d.fdst and f2; types, mass, fill levels, lists of the initial state
+// (walls: tmp may hold obstacle cells)
+void launch_init_state(const Dev &d, void *f2, const uint8_t *tmp, bool walls, cudaStream_t s);
 void launch_refresh(const Dev &d, cudaStream_t s);
 // f' = feq(rho, u) at the liquid and interface cells of the buffer d.fdst
 void launch_prescribe(const Dev &d, float rho, float ux, float uy, float uz, cudaStream_t s);
