@@ -360,94 +360,107 @@ __device__ T lsqr_core(const Acc &acc, uint8_t fi, T &cond_out) {
     full.init();
     red.init();
     const int kf = cons ? 3 : 5, kr = cons ? 1 : 3;
-    int m = 0;
-#pragma unroll 1
-    for (int dz = -1; dz <= 1; ++dz) {
-#pragma unroll 1
-        for (int t = 0; t < 9; ++t) {
-            const int dx = t % 3 - 1, dy = t / 3 - 1;
-            if (dx == 0 && dy == 0 && dz == 0) continue;
-            const uint8_t fj = acc.flag(dx, dy, dz);
-            if (!(fj & T_IF)) continue;
-            T nj[3], aj;
-            if (!acc.normal(dx, dy, dz, nj, aj)) continue;
-            const T o[3] = {T((double)dx), T((double)dy), T((double)dz)};
-            const T dv[3] = {o[0] + aj * nj[0] - p[0], o[1] + aj * nj[1] - p[1], o[2] + aj * nj[2] - p[2]};
-            const T u = dot3(dv, tu), v = dot3(dv, tv), f = dot3(dv, n);
-            if (!cons) {
-                T rf[5] = {u * u, v * v, u * v, u, v};
-                T rr[3] = {u * u + v * v, u, v};
-                full.add(rf, f, kf);
-                red.add(rr, f, kr);
-            } else {
-                const T rhs = f - gu * u - gv * v;
-                T rf[5] = {u * u - T(2) * uc * u, v * v - T(2) * vc * v, u * v - vc * u - uc * v, T(0), T(0)};
-                T rr[3] = {u * u + v * v - T(2) * uc * u - T(2) * vc * v, T(0), T(0)};
-                full.add(rf, rhs, kf);
-                red.add(rr, rhs, kr);
-            }
-            ++m;
-            if (fj & B_NEAR) {
-                T pc[3], mh[3];
-                if (!contact<T>(acc, dx, dy, dz, o, nj, aj, pc, mh)) continue;
-                const T mn = dot3(mh, n);
-                if (fabs(mn) < T(1e-6)) continue;
-                const T dc[3] = {pc[0] - p[0], pc[1] - p[1], pc[2] - p[2]};
-                const T uj = dot3(dc, tu), vj = dot3(dc, tv);
-                const T g1 = -dot3(mh, tu) / mn, g2 = -dot3(mh, tv) / mn;
-                if (!cons) {
-                    T r1[5] = {T(2) * uj, T(0), vj, T(1), T(0)};
-                    T r2[5] = {T(0), T(2) * vj, uj, T(0), T(1)};
-                    T s1[3] = {T(2) * uj, T(1), T(0)};
-                    T s2[3] = {T(2) * vj, T(0), T(1)};
-                    full.add(r1, g1, kf);
-                    full.add(r2, g2, kf);
-                    red.add(s1, g1, kr);
-                    red.add(s2, g2, kr);
-                } else {
-                    T r1[5] = {T(2) * (uj - uc), T(0), vj - vc, T(0), T(0)};
-                    T r2[5] = {T(0), T(2) * (vj - vc), uj - uc, T(0), T(0)};
-                    T s1[3] = {T(2) * (uj - uc), T(0), T(0)};
-                    T s2[3] = {T(2) * (vj - vc), T(0), T(0)};
-                    full.add(r1, g1 - gu, kf);
-                    full.add(r2, g2 - gv, kf);
-                    red.add(s1, g1 - gu, kr);
-                    red.add(s2, g2 - gv, kr);
-                }
-                m += 2;
-            }
-        }
-    }
     T A = T(0), B = T(0), C = T(0), H = T(0), I = T(0);
     T cond = T(1);
-    T sol[5] = {T(0), T(0), T(0), T(0), T(0)};
     bool done = false;
-    if (m >= kf && full.solve(sol, kf, cond)) {
-        A = sol[0];
-        B = sol[1];
-        C = sol[2];
-        if (cons) {
-            H = gu - T(2) * uc * A - vc * C;
-            I = gv - T(2) * vc * B - uc * C;
-        } else {
-            H = sol[3];
-            I = sol[4];
-        }
-        done = true;
-    } else {
-        T xr[3] = {T(0), T(0), T(0)};
-        T c2;
-        if (m >= kr && red.solve(xr, kr, c2)) {
-            cond = c2;
-            A = B = xr[0];
-            if (cons) {
-                H = gu - T(2) * uc * A;
-                I = gv - T(2) * vc * A;
-            } else {
-                H = xr[1];
-                I = xr[2];
+    // the full model; the isotropic one in a second pass only where that fails
+    // (both in one pass made the rotations of every fit 8 instead of 5 a row)
+#pragma unroll 1
+    for (int model = 0; model < 2 && !done; ++model) {
+        int m = 0;
+#pragma unroll 1
+        for (int dz = -1; dz <= 1; ++dz) {
+#pragma unroll 1
+            for (int t = 0; t < 9; ++t) {
+                const int dx = t % 3 - 1, dy = t / 3 - 1;
+                if (dx == 0 && dy == 0 && dz == 0) continue;
+                const uint8_t fj = acc.flag(dx, dy, dz);
+                if (!(fj & T_IF)) continue;
+                T nj[3], aj;
+                if (!acc.normal(dx, dy, dz, nj, aj)) continue;
+                const T o[3] = {T((double)dx), T((double)dy), T((double)dz)};
+                const T dv[3] = {o[0] + aj * nj[0] - p[0], o[1] + aj * nj[1] - p[1], o[2] + aj * nj[2] - p[2]};
+                const T u = dot3(dv, tu), v = dot3(dv, tv), f = dot3(dv, n);
+                if (!cons) {
+                    T rf[5] = {u * u, v * v, u * v, u, v};
+                    T rr[3] = {u * u + v * v, u, v};
+                    if (model == 0) full.add(rf, f, kf);
+                    else red.add(rr, f, kr);
+                } else {
+                    const T rhs = f - gu * u - gv * v;
+                    T rf[5] = {u * u - T(2) * uc * u, v * v - T(2) * vc * v, u * v - vc * u - uc * v, T(0), T(0)};
+                    T rr[3] = {u * u + v * v - T(2) * uc * u - T(2) * vc * v, T(0), T(0)};
+                    if (model == 0) full.add(rf, rhs, kf);
+                    else red.add(rr, rhs, kr);
+                }
+                ++m;
+                if (fj & B_NEAR) {
+                    T pc[3], mh[3];
+                    if (!contact<T>(acc, dx, dy, dz, o, nj, aj, pc, mh)) continue;
+                    const T mn = dot3(mh, n);
+                    if (fabs(mn) < T(1e-6)) continue;
+                    const T dc[3] = {pc[0] - p[0], pc[1] - p[1], pc[2] - p[2]};
+                    const T uj = dot3(dc, tu), vj = dot3(dc, tv);
+                    const T g1 = -dot3(mh, tu) / mn, g2 = -dot3(mh, tv) / mn;
+                    if (!cons) {
+                        T r1[5] = {T(2) * uj, T(0), vj, T(1), T(0)};
+                        T r2[5] = {T(0), T(2) * vj, uj, T(0), T(1)};
+                        T s1[3] = {T(2) * uj, T(1), T(0)};
+                        T s2[3] = {T(2) * vj, T(0), T(1)};
+                        if (model == 0) {
+                            full.add(r1, g1, kf);
+                            full.add(r2, g2, kf);
+                        } else {
+                            red.add(s1, g1, kr);
+                            red.add(s2, g2, kr);
+                        }
+                    } else {
+                        T r1[5] = {T(2) * (uj - uc), T(0), vj - vc, T(0), T(0)};
+                        T r2[5] = {T(0), T(2) * (vj - vc), uj - uc, T(0), T(0)};
+                        T s1[3] = {T(2) * (uj - uc), T(0), T(0)};
+                        T s2[3] = {T(2) * (vj - vc), T(0), T(0)};
+                        if (model == 0) {
+                            full.add(r1, g1 - gu, kf);
+                            full.add(r2, g2 - gv, kf);
+                        } else {
+                            red.add(s1, g1 - gu, kr);
+                            red.add(s2, g2 - gv, kr);
+                        }
+                    }
+                    m += 2;
+                }
             }
-            done = true;
+        }
+        if (model == 0) {
+            T sol[5] = {T(0), T(0), T(0), T(0), T(0)};
+            if (m >= kf && full.solve(sol, kf, cond)) {
+                A = sol[0];
+                B = sol[1];
+                C = sol[2];
+                if (cons) {
+                    H = gu - T(2) * uc * A - vc * C;
+                    I = gv - T(2) * vc * B - uc * C;
+                } else {
+                    H = sol[3];
+                    I = sol[4];
+                }
+                done = true;
+            }
+        } else {
+            T xr[3] = {T(0), T(0), T(0)};
+            T c2;
+            if (m >= kr && red.solve(xr, kr, c2)) {
+                cond = c2;
+                A = B = xr[0];
+                if (cons) {
+                    H = gu - T(2) * uc * A;
+                    I = gv - T(2) * vc * A;
+                } else {
+                    H = xr[1];
+                    I = xr[2];
+                }
+                done = true;
+            }
         }
     }
     cond_out = cond;
