@@ -202,10 +202,14 @@ int read_near(fsl_ctx *c) {
 }
 
 // enqueue the curvature of the current state into kappa_out
-void enqueue_curvature(const Dev &d, int model, float *kappa_out, cudaStream_t s) {
-    launch_normals(d, s);
+// (in_step: for the step's own use; fsl_curvature also leaves the normals)
+void enqueue_curvature(const Dev &d, int model, float *kappa_out, bool in_step, cudaStream_t s) {
+    // finite differences need no normals; the step reads them at contact lines
+    // and for normal-weighted excess shares
+    const bool normals = !in_step || model != FSL_CURV_FD || !d.inline_general || d.excess_rule;
+    if (normals) launch_normals(d, s);
     if (model == FSL_CURV_LSQR || model == FSL_CURV_MLP) launch_lsqr(d, kappa_out, s);
-    else if (model == FSL_CURV_FD) launch_fd(d, kappa_out, s);
+    else if (model == FSL_CURV_FD) launch_fd(d, kappa_out, !normals, s);
     else if (model == FSL_CURV_TR) launch_tr(d, kappa_out, s);
     else launch_zero_kappa(d, kappa_out, s);
     if (model == FSL_CURV_MLP) launch_mlp_curv(d, kappa_out, s);
@@ -228,7 +232,7 @@ int enqueue_step_graph(const fsl_ctx *c, int parity) {
         launch_normals(d, s);
         launch_curv_iface(d, s);
     } else {
-        enqueue_curvature(d, c->p.curv_model, d.kappa, s);
+        enqueue_curvature(d, c->p.curv_model, d.kappa, true, s);
         launch_sc_iface(d, s);
     }
     CK(cudaStreamWaitEvent(s, c->join, 0));
@@ -515,7 +519,7 @@ int fsl_step_profile(fsl_ctx *c, float ms_out[6]) {
         const bool fused = c->p.curv_model == FSL_CURV_LSQR;
         if (fused) launch_curv_iface(d, s);  // curvature + interface stream-collide
         else if (c->p.curv_model == FSL_CURV_MLP) launch_lsqr(d, d.kappa, s);
-        else if (c->p.curv_model == FSL_CURV_FD) launch_fd(d, d.kappa, s);
+        else if (c->p.curv_model == FSL_CURV_FD) launch_fd(d, d.kappa, false, s);
         else if (c->p.curv_model == FSL_CURV_TR) launch_tr(d, d.kappa, s);
         else launch_zero_kappa(d, d.kappa, s);
         if (c->p.curv_model == FSL_CURV_MLP) launch_mlp_curv(d, d.kappa, s);
@@ -541,7 +545,7 @@ int fsl_curvature(fsl_ctx *c, int model, float *kappa_out) {
     if (!c || !kappa_out || model < FSL_CURV_LSQR || model > FSL_CURV_TR) return FSL_EINVAL;
     if (model == FSL_CURV_MLP && !c->base.mlp_params) return FSL_EINVAL;
     const Dev d = dev_for(c, c->parity);
-    enqueue_curvature(d, model, kappa_out, c->stream);
+    enqueue_curvature(d, model, kappa_out, false, c->stream);
     return cudaGetLastError() == cudaSuccess ? FSL_OK : FSL_ECUDA;
 }
 

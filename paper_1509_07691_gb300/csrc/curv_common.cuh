@@ -197,6 +197,91 @@ __device__ __forceinline__ bool unit_normal_offset(T nv[3], T phi, int iters, T 
     return true;
 }
 
+// unit_normal_offset in FP32 with every rounding written out (which products
+// are fused is otherwise the compiler's choice, different from one caller to
+// the next): all kernels that form interface normals give the same bits.
+// al^3-type numerator of plic_vol_half, 3 al^2 - 3 al m1 + m1^2
+__device__ __forceinline__ float plic_base_rn(float al, float m1) {
+    const float p = __fmul_rn(3.0f, al);
+    return __fmaf_rn(m1, m1, __fmaf_rn(p, al, -__fmul_rn(p, m1)));
+}
+
+__device__ __forceinline__ float plic_vol_half_rn(float m1, float m2, float m3, float al) {
+    if (al < m1)
+        return __fdiv_rn(__fmul_rn(__fmul_rn(al, al), al), __fmul_rn(__fmul_rn(__fmul_rn(6.0f, m1), m2), m3));
+    const float den = __fmul_rn(__fmul_rn(6.0f, m2), m3);
+    float b = plic_base_rn(al, m1);
+    if (al < m2) return __fdiv_rn(b, den);
+    if (al >= __fadd_rn(m1, m2))
+        return __fdiv_rn(__fsub_rn(__fsub_rn(__fmul_rn(2.0f, al), m1), m2), __fmul_rn(2.0f, m3));
+    const float e2 = __fsub_rn(al, m2);
+    b = __fmaf_rn(-__fmul_rn(e2, e2), __fdiv_rn(e2, m1), b);
+    if (al >= m3) {
+        const float e3 = __fsub_rn(al, m3);
+        b = __fmaf_rn(-__fmul_rn(e3, e3), __fdiv_rn(e3, m1), b);
+    }
+    return __fdiv_rn(b, den);
+}
+
+__device__ __forceinline__ float plic_dvol_half_rn(float m1, float m2, float m3, float al) {
+    if (al < m1) return __fdiv_rn(__fmul_rn(al, al), __fmul_rn(__fmul_rn(__fmul_rn(2.0f, m1), m2), m3));
+    if (al < m2) return __fdiv_rn(__fsub_rn(__fmul_rn(2.0f, al), m1), __fmul_rn(__fmul_rn(2.0f, m2), m3));
+    if (al >= __fadd_rn(m1, m2)) return __fdiv_rn(1.0f, m3);
+    const float e2 = __fsub_rn(al, m2);
+    float t = __fmaf_rn(6.0f, al, -__fmul_rn(3.0f, m1));
+    t = __fmaf_rn(-__fmul_rn(3.0f, e2), __fdiv_rn(e2, m1), t);
+    if (al >= m3) {
+        const float e3 = __fsub_rn(al, m3);
+        t = __fmaf_rn(-__fmul_rn(3.0f, e3), __fdiv_rn(e3, m1), t);
+    }
+    return __fdiv_rn(t, __fmul_rn(__fmul_rn(6.0f, m2), m3));
+}
+
+__device__ __forceinline__ float4 plic_normal_rn(const float nv[3], float phi, int iters) {
+    const float l2 = __fmaf_rn(nv[2], nv[2], __fmaf_rn(nv[0], nv[0], __fmul_rn(nv[1], nv[1])));
+    if (!(l2 >= 1e-24f)) return make_float4(0.f, 0.f, 0.f, 0.f);
+    const float inv = rsqrtf(l2);
+    float4 n = make_float4(__fmul_rn(nv[0], inv), __fmul_rn(nv[1], inv), __fmul_rn(nv[2], inv), 0.f);
+    float a1 = fabsf(n.x), a2 = fabsf(n.y), a3 = fabsf(n.z), t;
+    const float M = __fadd_rn(__fadd_rn(a1, a2), a3);
+    if (phi <= 0.f || phi >= 1.f) {
+        n.w = phi <= 0.f ? 0.5f * M : -0.5f * M;
+        return n;
+    }
+    if (a1 > a2) { t = a1; a1 = a2; a2 = t; }
+    if (a2 > a3) { t = a2; a2 = a3; a3 = t; }
+    if (a1 > a2) { t = a1; a1 = a2; a2 = t; }
+    const float m1 = __fdiv_rn(a1, M), m2 = __fdiv_rn(a2, M), m3 = __fsub_rn(__fsub_rn(1.0f, m1), m2);
+    const bool mirror = phi > 0.5f;
+    const float v = mirror ? __fsub_rn(1.0f, phi) : phi;
+    const float den = __fmul_rn(__fmul_rn(6.0f, m2), m3);
+    const float V1 = m1 > 0.f ? __fdiv_rn(__fmul_rn(m1, m1), den) : 0.f;
+    const float V2 = m2 > 0.f ? __fdiv_rn(plic_base_rn(m2, m1), den) : 0.f;
+    const float s = __fadd_rn(m1, m2), c3 = fminf(m3, s);
+    const float V3 = plic_vol_half_rn(m1, m2, m3, c3);
+    float al;
+    if (v < V1) {
+        al = cbrtf(__fmul_rn(__fmul_rn(__fmul_rn(__fmul_rn(6.0f, m1), m2), m3), v));
+    } else if (v < V2) {
+        const float q = __fmaf_rn(__fmul_rn(__fmul_rn(72.0f, m2), m3), v, -__fmul_rn(__fmul_rn(3.0f, m1), m1));
+        al = __fadd_rn(__fmul_rn(0.5f, m1), __fmul_rn(__fsqrt_rn(fmaxf(q, 0.f)), 1.0f / 6.0f));
+    } else if (v >= V3 && m3 >= s) {
+        al = __fadd_rn(__fmul_rn(m3, v), __fmul_rn(0.5f, s));
+    } else {
+        const bool low = v < V3;
+        const float lo = low ? m2 : c3, hi = low ? c3 : 0.5f, vlo = low ? V2 : V3, vhi = low ? V3 : 0.5f;
+        al = vhi > vlo
+                 ? __fadd_rn(lo, __fdiv_rn(__fmul_rn(__fsub_rn(hi, lo), __fsub_rn(v, vlo)), __fsub_rn(vhi, vlo)))
+                 : lo;
+        for (int it = 0; it < iters; ++it) {
+            const float g = __fsub_rn(plic_vol_half_rn(m1, m2, m3, al), v);
+            al = fminf(fmaxf(__fsub_rn(al, __fdiv_rn(g, plic_dvol_half_rn(m1, m2, m3, al))), lo), hi);
+        }
+    }
+    n.w = __fmul_rn(M, __fsub_rn(0.5f, mirror ? __fsub_rn(1.0f, al) : al));
+    return n;
+}
+
 // ---- LSQR --------------------------------------------------------------------
 // Streaming Givens QR of a K-column least-squares problem (upper triangle R
 // and Q^T b kept in registers; rows are rotated in as they come).
@@ -469,6 +554,15 @@ __device__ T lsqr_core(const Acc &acc, uint8_t fi, T &cond_out) {
     return (A * (T(1) + I * I) + B * (T(1) + H * H) - C * H * I) / (g * sqrt(g));
 }
 
+// the FP64 re-solve of an ill-conditioned general fit; out of line, few cells take it
+template <typename Acc>
+__device__ __noinline__ float general_fit_fp64(const Dev &d, const Acc &acc, uint8_t fi) {
+    double cond;
+    const float kap = (float)lsqr_core<double>(acc, fi, cond);
+    atomicAdd(d.counts + C_FP64, 1);
+    return kap;
+}
+
 // Accessor of the forward kernels: flags and stored PLIC normals (float4
 // n, a) of the grid around cell (x, y, z); periodic wrap.
 struct GridAcc {
@@ -526,6 +620,173 @@ struct StagedAcc {
 __device__ __forceinline__ void stage_block(const Dev &d, int x, int y, int z, int lane, uint8_t *fl, float4 *nm) {
     for (int e = lane; e < 125; e += 32) fl[e] = d.flags[nbr_index(d, x, y, z, e % 5 - 2, (e / 5) % 5 - 2, e / 25 - 2)];
     if (lane < 27) nm[lane] = d.normal[nbr_index(d, x, y, z, lane % 3 - 1, (lane / 3) % 3 - 1, lane / 9 - 1)];
+}
+
+// The general fit of one cell by a warp, the arithmetic of lsqr_core<float>.
+// One lane alone is a chain of about 45 rows times 8 dependent Givens rotations
+// (square root, two divisions) behind 26 contact points: 41 us a launch.  Here
+//   lane t < 27 forms the rows of block cell t (point row, contact rows), which
+//     go to shared memory in lsqr_core's order;
+//   the rotations run as a pipeline: lane j holds row j of R and rotates row
+//     i of the fit into it while lane j + 1 rotates row i - 1; lanes 0..4 the
+//     full model, lanes 8..10 the isotropic one of the fallback;
+//   every lane solves.
+// 20 us a launch (cap of 7.4 k interface cells in 128 x 128 x 64).  cond as lsqr_core.  The whole warp must call it.
+constexpr int FIT_ROWS = 26 * 3;
+struct FitRows {
+    float full[FIT_ROWS][6], red[FIT_ROWS][4];  // coefficients, right-hand side
+};
+
+template <typename Acc>
+__device__ __forceinline__ float lsqr_warp(const Acc &acc, uint8_t fi, int lane, FitRows &rows, float &cond) {
+    const unsigned all = 0xffffffffu;
+    cond = 1.f;
+    float n[3], a;
+    if (!acc.normal(0, 0, 0, n, a)) return 0.f;  // warp-uniform
+    int k = 0;
+    if (fabsf(n[1]) < fabsf(n[0])) k = 1;
+    if (fabsf(n[2]) < fabsf(n[k])) k = 2;
+    float tu[3];
+    if (k == 0) { tu[0] = 0.f; tu[1] = -n[2]; tu[2] = n[1]; }
+    else if (k == 1) { tu[0] = n[2]; tu[1] = 0.f; tu[2] = -n[0]; }
+    else { tu[0] = -n[1]; tu[1] = n[0]; tu[2] = 0.f; }
+    const float tl = sqrtf(dot3(tu, tu));
+    tu[0] /= tl;
+    tu[1] /= tl;
+    tu[2] /= tl;
+    const float tv[3] = {n[1] * tu[2] - n[2] * tu[1], n[2] * tu[0] - n[0] * tu[2], n[0] * tu[1] - n[1] * tu[0]};
+    const float p[3] = {a * n[0], a * n[1], a * n[2]};
+    // this lane's block cell: point, contact point
+    const int t = lane < 27 ? lane : 13, dx = t % 3 - 1, dy = (t / 3) % 3 - 1, dz = t / 9 - 1;
+    const uint8_t fj = t == 13 ? fi : acc.flag(dx, dy, dz);
+    float nj[3] = {0.f, 0.f, 0.f}, aj = 0.f;
+    const bool have = lane < 27 && ((fj & T_IF) || t == 13) && acc.normal(dx, dy, dz, nj, aj);
+    const bool point = have && t != 13;
+    const float o[3] = {(float)dx, (float)dy, (float)dz};
+    const float dv[3] = {o[0] + aj * nj[0] - p[0], o[1] + aj * nj[1] - p[1], o[2] + aj * nj[2] - p[2]};
+    const float u = dot3(dv, tu), v = dot3(dv, tv), f = dot3(dv, n);
+    bool touch = false;
+    float uj = 0.f, vj = 0.f, g1 = 0.f, g2 = 0.f;
+    if (have && (fj & B_NEAR)) {
+        float pc[3], mh[3];
+        if (contact<float>(acc, dx, dy, dz, o, nj, aj, pc, mh)) {
+            const float mn = dot3(mh, n);
+            if (fabsf(mn) >= 1e-6f) {
+                const float dc[3] = {pc[0] - p[0], pc[1] - p[1], pc[2] - p[2]};
+                uj = dot3(dc, tu);
+                vj = dot3(dc, tv);
+                g1 = -dot3(mh, tu) / mn;
+                g2 = -dot3(mh, tv) / mn;
+                touch = true;
+            }
+        }
+    }
+    // the centre's contact point constrains the gradient there
+    const bool cons = __shfl_sync(all, touch ? 1 : 0, 13) != 0;
+    const float uc = __shfl_sync(all, uj, 13), vc = __shfl_sync(all, vj, 13);
+    const float gu = __shfl_sync(all, g1, 13), gv = __shfl_sync(all, g2, 13);
+    const unsigned pm = __ballot_sync(all, point), tm = __ballot_sync(all, point && touch);
+    const unsigned lt = (1u << lane) - 1u;
+    const int m = __popc(pm) + 2 * __popc(tm);
+    int at = __popc(pm & lt) + 2 * __popc(tm & lt);
+    auto put = [&](float a0, float a1, float a2, float a3, float a4, float r0, float r1, float r2, float b) {
+        float *q = rows.full[at], *r = rows.red[at];
+        q[0] = a0; q[1] = a1; q[2] = a2; q[3] = a3; q[4] = a4; q[5] = b;
+        r[0] = r0; r[1] = r1; r[2] = r2; r[3] = b;
+        ++at;
+    };
+    if (point) {
+        if (!cons) {
+            put(u * u, v * v, u * v, u, v, u * u + v * v, u, v, f);
+            if (touch) {
+                put(2.f * uj, 0.f, vj, 1.f, 0.f, 2.f * uj, 1.f, 0.f, g1);
+                put(0.f, 2.f * vj, uj, 0.f, 1.f, 2.f * vj, 0.f, 1.f, g2);
+            }
+        } else {
+            put(u * u - 2.f * uc * u, v * v - 2.f * vc * v, u * v - vc * u - uc * v, 0.f, 0.f,
+                u * u + v * v - 2.f * uc * u - 2.f * vc * v, 0.f, 0.f, f - gu * u - gv * v);
+            if (touch) {
+                put(2.f * (uj - uc), 0.f, vj - vc, 0.f, 0.f, 2.f * (uj - uc), 0.f, 0.f, g1 - gu);
+                put(0.f, 2.f * (vj - vc), uj - uc, 0.f, 0.f, 2.f * (vj - vc), 0.f, 0.f, g2 - gv);
+            }
+        }
+    }
+    __syncwarp();
+    // pipelined Givens rotations
+    const int j = lane & 7, kf = cons ? 3 : 5, kr = cons ? 1 : 3;
+    const int cols = lane < 8 ? kf : (lane < 16 ? kr : 0);
+    float R[5] = {0.f, 0.f, 0.f, 0.f, 0.f}, qb = 0.f, w[5] = {0.f, 0.f, 0.f, 0.f, 0.f}, b = 0.f;
+    for (int it = 0; it < m + 4; ++it) {
+        // the row: from shared memory for column 0, else what the column before made of it
+#pragma unroll
+        for (int l = 0; l < 4; ++l) w[l] = __shfl_up_sync(all, w[l + 1], 1);
+        b = __shfl_up_sync(all, b, 1);
+        if (j == 0) {
+            const int r = min(it, FIT_ROWS - 1);
+            if (lane == 0) {
+#pragma unroll
+                for (int l = 0; l < 5; ++l) w[l] = rows.full[r][l];
+                b = rows.full[r][5];
+            } else {
+#pragma unroll
+                for (int l = 0; l < 3; ++l) w[l] = rows.red[r][l];
+                w[3] = w[4] = 0.f;
+                b = rows.red[r][3];
+            }
+        } else {
+            w[4] = 0.f;
+        }
+        if (j < cols && it >= j && it - j < m) {
+            const float h = sqrtf(R[0] * R[0] + w[0] * w[0]);
+            if (h != 0.f) {
+                const float c = R[0] / h, s = w[0] / h;
+                R[0] = h;
+#pragma unroll
+                for (int l = 1; l < 5; ++l) {
+                    const float r = R[l];
+                    R[l] = c * r + s * w[l];
+                    w[l] = c * w[l] - s * r;
+                }
+                const float z = qb;
+                qb = c * z + s * b;
+                b = c * b - s * z;
+            }
+        }
+    }
+    Givens<float, 5> full;
+    Givens<float, 3> red;
+#pragma unroll
+    for (int r = 0; r < 5; ++r) {
+#pragma unroll
+        for (int c = r; c < 5; ++c) full.R[Givens<float, 5>::at(r, c)] = __shfl_sync(all, R[c - r], r);
+        full.qb[r] = __shfl_sync(all, qb, r);
+    }
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+#pragma unroll
+        for (int c = r; c < 3; ++c) red.R[Givens<float, 3>::at(r, c)] = __shfl_sync(all, R[c - r], 8 + r);
+        red.qb[r] = __shfl_sync(all, qb, 8 + r);
+    }
+    __syncwarp();
+    float A, B, C, H, I, sol[5] = {0.f, 0.f, 0.f, 0.f, 0.f}, c2;
+    if (m >= kf && full.solve(sol, kf, c2)) {
+        A = sol[0];
+        B = sol[1];
+        C = sol[2];
+        H = cons ? gu - 2.f * uc * A - vc * C : sol[3];
+        I = cons ? gv - 2.f * vc * B - uc * C : sol[4];
+    } else {
+        float xr[3] = {0.f, 0.f, 0.f};
+        if (m >= kf) cond = c2;  // the full model's, as lsqr_core reports a fit it could not take
+        if (!(m >= kr && red.solve(xr, kr, c2))) return 0.f;
+        A = B = xr[0];
+        C = 0.f;
+        H = cons ? gu - 2.f * uc * A : xr[1];
+        I = cons ? gv - 2.f * vc * A : xr[2];
+    }
+    cond = c2;
+    const float g = 1.f + H * H + I * I;
+    return (A * (1.f + I * I) + B * (1.f + H * H) - C * H * I) / (g * sqrtf(g));
 }
 
 // Fast path: FP32 normal equations of the full model for an interface cell

@@ -377,7 +377,8 @@ void launch_convert(const Dev &d, cudaStream_t s);
 void launch_finalize(const Dev &d, cudaStream_t s);
 void launch_normals(const Dev &d, cudaStream_t s);
 void launch_lsqr(const Dev &d, float *kappa_out, cudaStream_t s);
-void launch_fd(const Dev &d, float *kappa_out, cudaStream_t s);
+// first: nothing of the pass has run before (the normals are needed by walls only)
+void launch_fd(const Dev &d, float *kappa_out, bool first, cudaStream_t s);
 void launch_tr(const Dev &d, float *kappa_out, cudaStream_t s);
 void launch_zero_kappa(const Dev &d, float *kappa_out, cudaStream_t s);
 void launch_mlp_curv(const Dev &d, float *kappa_out, cudaStream_t s);

@@ -17,19 +17,75 @@ namespace fslk {
 
 constexpr int LIST_THREADS = 128;
 
+// Parker-Youngs gradient of a cell next to an obstacle, by a warp: lane t takes
+// block cell t, reflecting the fill level of an obstacle cell (Sec. II.A; two
+// rounds of loads each), and the 27 values are handed round.
+__device__ __forceinline__ void gradient_near_wall(const Dev &d, int i, int lane, float nv[3]) {
+    int x, y, z;
+    cell_coords(d, i, x, y, z);
+    const int t = lane < 27 ? lane : 13;
+    const float v = phi_ext(d, x + t % 3 - 1, y + (t / 3) % 3 - 1, z + t / 9 - 1);
+    float ph[27];
+#pragma unroll
+    for (int e = 0; e < 27; ++e) ph[e] = __shfl_sync(0xffffffffu, v, e);
+    parker_youngs<float>([&](int dx, int dy, int dz) { return ph[(dz + 1) * 9 + (dy + 1) * 3 + (dx + 1)]; }, nv);
+}
+
+// One thread per interface cell.  Cells next to an obstacle come in rounds of
+// their own: their gradients take nine or more reflections, which one thread ran
+// one after another (24 us a launch for the cap of 7.4 k interface cells in
+// 128 x 128 x 64, 11 us now), so the warp forms each of them together.  They follow
+// one another in the list (the layer at the wall), so there the lanes of a warp
+// look at entries far apart.
 // The first kernel of a step also runs the step prologue (counters, bubble
 // pressure); every later kernel of the step is ordered after it on the stream.
-__global__ void __launch_bounds__(LIST_THREADS) k_normals(Dev d) {
+__global__ void __launch_bounds__(LIST_THREADS) k_normals(const __grid_constant__ Dev d) {
     pdl_enter();
     int cnt[1];
     block_counts<1>(d.counts, {d.cif}, cnt);
     const int n = cnt[0];
     if (blockIdx.x == 0 && threadIdx.x == 0) step_prologue(d);
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x)
-        normal_cell(d, d.iflist[k]);
+    const int lane = threadIdx.x & 31, nth = gridDim.x * blockDim.x, nw = nth >> 5;
+    const int tid = blockIdx.x * blockDim.x + threadIdx.x, gw = tid >> 5;
+    const int rounds = (n + nth - 1) / nth;
+    for (int r = 0; r < (d.inline_general ? rounds : 2 * rounds); ++r) {  // warp-uniform
+        const bool walls = r >= rounds;
+        const int k = walls ? (r - rounds) * nth + lane * nw + gw : r * nth + tid;
+        bool mine = k < n;
+        const int i = mine ? d.iflist[k] : 0;
+        float nv[3] = {0.f, 0.f, 0.f}, phi = 0.f;
+        if (!walls) {
+            if (mine) {
+                int x, y, z;
+                cell_coords(d, i, x, y, z);
+                // the 27 fill levels are loaded with the cell's type (one round)
+                float ph[27];
+#pragma unroll
+                for (int t = 0; t < 27; ++t) ph[t] = d.phi[nbr_index(d, x, y, z, t % 3 - 1, (t / 3) % 3 - 1, t / 9 - 1)];
+                mine = !(d.flags[i] & B_NEAR);
+                parker_youngs<float>([&](int dx, int dy, int dz) { return ph[(dz + 1) * 9 + (dy + 1) * 3 + (dx + 1)]; }, nv);
+                phi = ph[13];
+            }
+        } else {
+            mine = mine && (d.flags[i] & B_NEAR);
+            if (mine) phi = d.phi[i];
+            for (unsigned near = __ballot_sync(0xffffffffu, mine); near; near &= near - 1u) {
+                const int who = __ffs(near) - 1;
+                float g[3];
+                gradient_near_wall(d, __shfl_sync(0xffffffffu, i, who), lane, g);
+                if (lane == who) {
+                    nv[0] = g[0];
+                    nv[1] = g[1];
+                    nv[2] = g[2];
+                }
+            }
+        }
+        if (mine) d.normal[i] = plic_normal_rn(nv, phi, d.plic_iters);
+    }
 }
 
 __global__ void __launch_bounds__(LIST_THREADS) k_lsqr_fast(Dev d, float *kappa_out) {
+    pdl_enter();
     int cnt[1];
     block_counts<1>(d.counts, {d.cif}, cnt);
     const int n = cnt[0];
@@ -50,32 +106,27 @@ __global__ void __launch_bounds__(LIST_THREADS) k_lsqr_fast(Dev d, float *kappa_
 
 // General path: contact rows and centre constraint, isotropic fallback, FP64
 // re-solve when the FP32 R is ill conditioned
-__global__ void __launch_bounds__(LIST_THREADS) k_lsqr_slow(Dev d, float *kappa_out) {
+__global__ void __launch_bounds__(LIST_THREADS) k_lsqr_slow(const __grid_constant__ Dev d, float *kappa_out) {
     __shared__ uint8_t sfl[LIST_THREADS / 32][128];
     __shared__ float4 snm[LIST_THREADS / 32][27];
+    __shared__ FitRows rows[LIST_THREADS / 32];
+    pdl_enter();
     int cnt[1];
     block_counts<1>(d.counts, {C_SLOW}, cnt);
     const int n = cnt[0];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), nw = (int)((gridDim.x * blockDim.x) >> 5);
-    for (int k = gw; k < n; k += nw) {  // warp per cell: the block staged, one lane fits
+    for (int k = gw; k < n; k += nw) {  // warp per cell, its block staged
         const int i = d.slow[k];
         int x, y, z;
         cell_coords(d, i, x, y, z);
         stage_block(d, x, y, z, lane, sfl[w], snm[w]);
         __syncwarp();
-        if (lane == 0) {
-            const StagedAcc acc{d, sfl[w], snm[w]};
-            const uint8_t fi = d.flags[i];
-            float cond;
-            float kap = lsqr_core<float>(acc, fi, cond);
-            if (cond * cond > d.fp64_cond) {
-                double c2;
-                kap = (float)lsqr_core<double>(acc, fi, c2);
-                atomicAdd(d.counts + C_FP64, 1);
-            }
-            kappa_out[i] = kap;
-        }
+        const StagedAcc acc{d, sfl[w], snm[w]};
+        const uint8_t fi = d.flags[i];
+        float cond;
+        const float kap = lsqr_warp(acc, fi, lane, rows[w], cond);
+        if (lane == 0) kappa_out[i] = cond * cond > d.fp64_cond ? general_fit_fp64(d, acc, fi) : kap;
         __syncwarp();
     }
 }
@@ -98,6 +149,7 @@ constexpr float TR_TWO_PI = 6.28318530717958647692f;
 constexpr float TR_PI = 3.14159265358979323846f;
 
 __global__ void __launch_bounds__(LIST_THREADS) k_tr(Dev d, float *kappa_out) {
+    pdl_enter();
     int cnt[1];
     block_counts<1>(d.counts, {d.cif}, cnt);
     const int n = cnt[0];
@@ -265,13 +317,47 @@ __device__ __noinline__ float fd_cell(const Dev &d, int x, int y, int z) {
     return -0.25f * div;
 }
 
-__global__ void __launch_bounds__(32 * FD_WARPS) k_fd_warp(Dev d, float *kappa_out) {
+// The stencil in reach of the six normals: 81 smoothed values (offsets in
+// -2..2, at most one of them +-2) from 275 fill levels (-3..3, at most one
+// +-3), as packed places x + 7 y + 49 z of the 7^3 block.
+struct FdTable {
+    uint16_t phi[275];
+    uint8_t sm[81], pad;
+};
+constexpr FdTable fd_table() {
+    FdTable t{};
+    int np = 0, ns = 0;
+    for (int z = -3; z <= 3; ++z)
+        for (int y = -3; y <= 3; ++y)
+            for (int x = -3; x <= 3; ++x) {
+                const int far = (x * x == 9) + (y * y == 9) + (z * z == 9);
+                const int mid = (x * x == 4) + (y * y == 4) + (z * z == 4);
+                if (far <= 1) t.phi[np++] = (uint16_t)((z + 3) * 49 + (y + 3) * 7 + x + 3);
+                if (far == 0 && mid <= 1) t.sm[ns++] = (uint8_t)((z + 2) * 25 + (y + 2) * 5 + x + 2);
+            }
+    return t;
+}
+__constant__ FdTable FD_TABLE = fd_table();
+
+// WALLS: the domain has obstacle cells (k_normals has run before); without
+// them no cell types are read, only the 275 fill levels are staged, and the
+// registers of the wall path do not hold down the resident warps: 66 -> 40 us
+// for 28.6 k interface cells.  prologue: this kernel comes first and runs the
+// step prologue.
+template <bool WALLS>
+__global__ void __launch_bounds__(32 * FD_WARPS) k_fd_warp(const __grid_constant__ Dev d, float *kappa_out, int prologue) {
     __shared__ float s_phi[FD_WARPS][343];
     __shared__ float s_sm[FD_WARPS][125];
     __shared__ float s_n[FD_WARPS][6][3];
+    __shared__ FdTable tab;
+    pdl_enter();
+    if (!WALLS)
+        for (int e = threadIdx.x; e < (int)(sizeof(FdTable) / 2); e += blockDim.x)
+            reinterpret_cast<uint16_t *>(&tab)[e] = reinterpret_cast<const uint16_t *>(&FD_TABLE)[e];
     int cnt[1];
-    block_counts<1>(d.counts, {d.cif}, cnt);
+    block_counts<1>(d.counts, {d.cif}, cnt);  // synchronises the block
     const int n = cnt[0];
+    if (prologue && blockIdx.x == 0 && threadIdx.x == 0) step_prologue(d);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), nw = (int)((gridDim.x * blockDim.x) >> 5);
     float *ph = s_phi[w], *sm = s_sm[w];
@@ -279,26 +365,41 @@ __global__ void __launch_bounds__(32 * FD_WARPS) k_fd_warp(Dev d, float *kappa_o
         const int i = d.iflist[k];
         int x, y, z;
         cell_coords(d, i, x, y, z);
-        bool obs = false;
-        for (int e = lane; e < 343; e += 32) {
-            const int j = nbr_index(d, x, y, z, e % 7 - 3, (e / 7) % 7 - 3, e / 49 - 3);
-            obs |= (d.flags[j] & T_OBS) != 0;
-            ph[e] = d.phi[j];
-        }
-        if (__any_sync(0xffffffffu, obs)) {  // walls in reach: the per-cell path
-            if (lane == 0) kappa_out[i] = fd_cell(d, x, y, z);
-            __syncwarp();
-            continue;
+        if (WALLS) {
+            bool obs = false;
+            for (int e = lane; e < 343; e += 32) {
+                const int j = nbr_index(d, x, y, z, e % 7 - 3, (e / 7) % 7 - 3, e / 49 - 3);
+                obs |= (d.flags[j] & T_OBS) != 0;
+                ph[e] = d.phi[j];
+            }
+            if (__any_sync(0xffffffffu, obs)) {  // walls in reach: the per-cell path
+                if (lane == 0) kappa_out[i] = fd_cell(d, x, y, z);
+                __syncwarp();
+                continue;
+            }
+        } else {
+#pragma unroll
+            for (int t = 0; t < 9; ++t) {
+                const int q = lane + 32 * t;
+                if (q < 275) {
+                    const int e = tab.phi[q];
+                    ph[e] = d.phi[nbr_index(d, x, y, z, e % 7 - 3, (e / 7) % 7 - 3, e / 49 - 3)];
+                }
+            }
         }
         __syncwarp();
         // smoothed fill level of the 5^3 block (offsets -2..2), as smooth_at
-        for (int e = lane; e < 125; e += 32) {
+        for (int q = lane; q < (WALLS ? 125 : 81); q += 32) {
+            const int e = WALLS ? q : tab.sm[q];
             const int ex = e % 5 + 1, ey = (e / 5) % 5 + 1, ez = e / 25 + 1;  // in the 7^3 block
             float acc = 0.f;
+#pragma unroll
             for (int dz = -1; dz <= 1; ++dz)
+#pragma unroll
                 for (int dy = -1; dy <= 1; ++dy)
+#pragma unroll
                     for (int dx = -1; dx <= 1; ++dx)
-                        acc += k8w(dx, dy, dz) * ph[(ez + dz) * 49 + (ey + dy) * 7 + ex + dx];
+                        acc = fmaf(k8w(dx, dy, dz), ph[(ez + dz) * 49 + (ey + dy) * 7 + ex + dx], acc);
             sm[e] = acc * (1.0f / 3.6796875f);
         }
         __syncwarp();
@@ -340,16 +441,19 @@ void launch_normals(const Dev &d, cudaStream_t s) {
 void launch_lsqr(const Dev &d, float *kappa_out, cudaStream_t s) {
     static const int gf = list_blocks((const void *)k_lsqr_fast, LIST_THREADS, 4);
     static const int gs = list_blocks((const void *)k_lsqr_slow, LIST_THREADS, 4);
-    k_lsqr_fast<<<gf, LIST_THREADS, 0, s>>>(d, kappa_out);
-    k_lsqr_slow<<<gs, LIST_THREADS, 0, s>>>(d, kappa_out);
+    launch_pdl(k_lsqr_fast, gf, LIST_THREADS, s, d, kappa_out);
+    launch_pdl(k_lsqr_slow, gs, LIST_THREADS, s, d, kappa_out);
 }
-void launch_fd(const Dev &d, float *kappa_out, cudaStream_t s) {
-    static const int g = list_blocks((const void *)k_fd_warp, 32 * FD_WARPS, 16);
-    k_fd_warp<<<g, 32 * FD_WARPS, 0, s>>>(d, kappa_out);
+void launch_fd(const Dev &d, float *kappa_out, bool first, cudaStream_t s) {
+    static const int g = list_blocks((const void *)k_fd_warp<true>, 32 * FD_WARPS, 16);
+    static const int g0 = list_blocks((const void *)k_fd_warp<false>, 32 * FD_WARPS, 16);
+    if (!d.inline_general) launch_pdl(k_fd_warp<true>, g, 32 * FD_WARPS, s, d, kappa_out, 0);
+    else if (first) k_fd_warp<false><<<g0, 32 * FD_WARPS, 0, s>>>(d, kappa_out, 1);
+    else launch_pdl(k_fd_warp<false>, g0, 32 * FD_WARPS, s, d, kappa_out, 0);
 }
 void launch_tr(const Dev &d, float *kappa_out, cudaStream_t s) {
     static const int g = list_blocks((const void *)k_tr, LIST_THREADS, 8);
-    k_tr<<<g, LIST_THREADS, 0, s>>>(d, kappa_out);
+    launch_pdl(k_tr, g, LIST_THREADS, s, d, kappa_out);
 }
 void launch_zero_kappa(const Dev &d, float *kappa_out, cudaStream_t s) {
     static const int g = list_blocks((const void *)k_zero_kappa, LIST_THREADS, 4);

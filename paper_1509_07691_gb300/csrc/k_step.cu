@@ -32,6 +32,7 @@ __global__ void __launch_bounds__(256, S == FSL_F32 ? 5 : 4) k_sc_bulk(Dev d) {
 
 template <int S, int COLL>
 __global__ void __launch_bounds__(LIST_BLOCK) k_sc_iface(Dev d) {
+    pdl_enter();
     int cnt[1];
     block_counts<1>(d.counts, {d.cif}, cnt);
     const int n = cnt[0];
@@ -82,14 +83,19 @@ __global__ void __launch_bounds__(LIST_BLOCK, IFACE_MIN_BLOCKS) k_curv_iface_fas
 }
 
 // General-path cells (contact-line cells, degenerate or ill-conditioned FP32
-// fits): one warp per cell stages the block in shared memory, then one lane
-// runs the streaming Givens fit (FP64 when ill conditioned) and the
-// interface stream-collide of the cell.
-template <int S, int COLL>
-__global__ void __launch_bounds__(LIST_BLOCK) k_curv_iface_slow(Dev d) {
+// fits): one warp per cell stages the block in shared memory and runs the
+// Givens fit as a pipeline over its lanes (lsqr_warp; FP64 by one lane when
+// ill conditioned), then one lane the interface stream-collide of the cell.
+// PIPE: the fit by lsqr_warp; else lsqr_core by one lane.  The two differ in
+// which products are fused (kappa by about 1e-7), and a window's gradients
+// magnify the last bits of its states near full and empty cells, so the frozen
+// steps of a window keep the one-lane order.
+template <int S, int COLL, bool PIPE>
+__global__ void __launch_bounds__(LIST_BLOCK) k_curv_iface_slow(const __grid_constant__ Dev d) {
     pdl_enter();
     __shared__ uint8_t sfl[LIST_BLOCK / 32][128];
     __shared__ float4 snm[LIST_BLOCK / 32][27];
+    __shared__ FitRows rows[LIST_BLOCK / 32];
     int cnt[1];
     block_counts<1>(d.counts, {C_SLOW}, cnt);
     const int n = cnt[0];
@@ -101,7 +107,19 @@ __global__ void __launch_bounds__(LIST_BLOCK) k_curv_iface_slow(Dev d) {
         cell_coords(d, i, x, y, z);
         stage_block(d, x, y, z, lane, sfl[w], snm[w]);
         __syncwarp();
-        if (lane == 0) general_cell<S, COLL>(d, StagedAcc{d, sfl[w], snm[w]}, i);
+        const StagedAcc acc{d, sfl[w], snm[w]};
+        if (PIPE) {
+            const uint8_t fi = d.flags[i] & (T_MASK | B_NEAR);
+            float cond;
+            float kap = lsqr_warp(acc, fi, lane, rows[w], cond);
+            if (lane == 0) {
+                if (cond * cond > d.fp64_cond) kap = general_fit_fp64(d, acc, fi);
+                d.kappa[i] = kap;
+                iface_cell<S, COLL>(d, i);
+            }
+        } else if (lane == 0) {
+            general_cell<S, COLL>(d, acc, i);
+        }
         __syncwarp();
     }
 }
@@ -213,7 +231,7 @@ void launch_bulk(const Dev &d, cudaStream_t s) {
 template <int S, int COLL>
 void launch_iface(const Dev &d, cudaStream_t s) {
     static const int gi = list_blocks((const void *)k_sc_iface<S, COLL>, LIST_BLOCK, 4);
-    k_sc_iface<S, COLL><<<gi, LIST_BLOCK, 0, s>>>(d);
+    launch_pdl(k_sc_iface<S, COLL>, gi, LIST_BLOCK, s, d);
 }
 
 #define FSL_DISPATCH(FN)                                                                          \
@@ -229,9 +247,12 @@ void launch_iface(const Dev &d, cudaStream_t s) {
 template <int S, int COLL>
 void launch_ci(const Dev &d, cudaStream_t s) {
     static const int gf = list_blocks((const void *)k_curv_iface_fast<S, COLL, FSL_IFACE_LANES>, LIST_BLOCK, 4);
-    static const int gs = list_blocks((const void *)k_curv_iface_slow<S, COLL>, LIST_BLOCK, 4);
+    static const int gs = list_blocks((const void *)k_curv_iface_slow<S, COLL, true>, LIST_BLOCK, 4);
+    static const int gz = list_blocks((const void *)k_curv_iface_slow<S, COLL, false>, LIST_BLOCK, 4);
     launch_pdl(k_curv_iface_fast<S, COLL, FSL_IFACE_LANES>, gf, LIST_BLOCK, s, d);
-    if (!d.inline_general) launch_pdl(k_curv_iface_slow<S, COLL>, gs, LIST_BLOCK, s, d);
+    if (d.inline_general) return;
+    if (d.frozen) launch_pdl(k_curv_iface_slow<S, COLL, false>, gz, LIST_BLOCK, s, d);
+    else launch_pdl(k_curv_iface_slow<S, COLL, true>, gs, LIST_BLOCK, s, d);
 }
 
 void launch_sc_bulk(const Dev &d, cudaStream_t s) { FSL_DISPATCH(launch_bulk); }

@@ -8,31 +8,6 @@
 
 namespace fslk {
 
-// Parker-Youngs normal of a cell next to an obstacle (reflected fill levels at
-// the obstacle cells); out of line, so that the loop of k_normals stays short
-static __device__ __noinline__ void normal_near_wall(const Dev &d, int x, int y, int z, float nv[3]) {
-    parker_youngs<float>([&](int dx, int dy, int dz) { return phi_ext(d, x + dx, y + dy, z + dz); }, nv);
-}
-
-// normal and PLIC offset of interface cell i
-__device__ __forceinline__ void normal_cell(const Dev &d, int i) {
-    int x, y, z;
-    cell_coords(d, i, x, y, z);
-    // the 27 fill levels are loaded with the cell's type (one round); a cell
-    // next to a wall takes the reflected ones instead, out of line
-    float ph[27];
-#pragma unroll
-    for (int t = 0; t < 27; ++t) ph[t] = d.phi[nbr_index(d, x, y, z, t % 3 - 1, (t / 3) % 3 - 1, t / 9 - 1)];
-    const uint8_t fl = d.flags[i];
-    float nv[3], a;
-    if (fl & B_NEAR)
-        normal_near_wall(d, x, y, z, nv);
-    else
-        parker_youngs<float>([&](int dx, int dy, int dz) { return ph[(dz + 1) * 9 + (dy + 1) * 3 + (dx + 1)]; }, nv);
-    const bool ok = unit_normal_offset<float>(nv, ph[13], d.plic_iters, a);
-    d.normal[i] = ok ? make_float4(nv[0], nv[1], nv[2], a) : make_float4(0.f, 0.f, 0.f, 0.f);
-}
-
 // index of the source cell x - c_q of every direction
 __device__ __forceinline__ void sources(const Dev &d, int x, int y, int z, int src[Q]) {
     const int xs[3] = {x == d.nx - 1 ? 0 : x + 1, x, x == 0 ? d.nx - 1 : x - 1};  // x - c for c = -1, 0, 1
@@ -220,11 +195,7 @@ __device__ __forceinline__ void general_cell(const Dev &d, const Acc &acc, int i
     const uint8_t fi = d.flags[i] & (T_MASK | B_NEAR);
     float cond;
     float kap = lsqr_core<float>(acc, fi, cond);
-    if (cond * cond > d.fp64_cond) {
-        double c2;
-        kap = (float)lsqr_core<double>(acc, fi, c2);
-        atomicAdd(d.counts + C_FP64, 1);
-    }
+    if (cond * cond > d.fp64_cond) kap = general_fit_fp64(d, acc, fi);
     d.kappa[i] = kap;
     iface_cell<S, COLL>(d, i);
 }
