@@ -633,46 +633,51 @@ __device__ __forceinline__ void stage_block(const Dev &d, int x, int y, int z, i
 //   every lane solves.
 // 20 us a launch (cap of 7.4 k interface cells in 128 x 128 x 64).  cond as lsqr_core.  The whole warp must call it.
 constexpr int FIT_ROWS = 26 * 3;
-struct FitRows {
-    float full[FIT_ROWS][6], red[FIT_ROWS][4];  // coefficients, right-hand side
+template <typename T>
+struct FitRowsOf {
+    T full[FIT_ROWS][6], red[FIT_ROWS][4];  // coefficients, right-hand side
+};
+union FitRows {
+    FitRowsOf<float> f;
+    FitRowsOf<double> d;
 };
 
-template <typename Acc>
-__device__ __forceinline__ float lsqr_warp(const Acc &acc, uint8_t fi, int lane, FitRows &rows, float &cond) {
+template <typename T, typename Acc>
+__device__ __forceinline__ T lsqr_warp(const Acc &acc, uint8_t fi, int lane, FitRowsOf<T> &rows, T &cond) {
     const unsigned all = 0xffffffffu;
-    cond = 1.f;
-    float n[3], a;
-    if (!acc.normal(0, 0, 0, n, a)) return 0.f;  // warp-uniform
+    cond = T(1);
+    T n[3], a;
+    if (!acc.normal(0, 0, 0, n, a)) return T(0);  // warp-uniform
     int k = 0;
-    if (fabsf(n[1]) < fabsf(n[0])) k = 1;
-    if (fabsf(n[2]) < fabsf(n[k])) k = 2;
-    float tu[3];
-    if (k == 0) { tu[0] = 0.f; tu[1] = -n[2]; tu[2] = n[1]; }
-    else if (k == 1) { tu[0] = n[2]; tu[1] = 0.f; tu[2] = -n[0]; }
-    else { tu[0] = -n[1]; tu[1] = n[0]; tu[2] = 0.f; }
-    const float tl = sqrtf(dot3(tu, tu));
+    if (fabs(n[1]) < fabs(n[0])) k = 1;
+    if (fabs(n[2]) < fabs(n[k])) k = 2;
+    T tu[3];
+    if (k == 0) { tu[0] = T(0); tu[1] = -n[2]; tu[2] = n[1]; }
+    else if (k == 1) { tu[0] = n[2]; tu[1] = T(0); tu[2] = -n[0]; }
+    else { tu[0] = -n[1]; tu[1] = n[0]; tu[2] = T(0); }
+    const T tl = sqrt(dot3(tu, tu));
     tu[0] /= tl;
     tu[1] /= tl;
     tu[2] /= tl;
-    const float tv[3] = {n[1] * tu[2] - n[2] * tu[1], n[2] * tu[0] - n[0] * tu[2], n[0] * tu[1] - n[1] * tu[0]};
-    const float p[3] = {a * n[0], a * n[1], a * n[2]};
+    const T tv[3] = {n[1] * tu[2] - n[2] * tu[1], n[2] * tu[0] - n[0] * tu[2], n[0] * tu[1] - n[1] * tu[0]};
+    const T p[3] = {a * n[0], a * n[1], a * n[2]};
     // this lane's block cell: point, contact point
     const int t = lane < 27 ? lane : 13, dx = t % 3 - 1, dy = (t / 3) % 3 - 1, dz = t / 9 - 1;
     const uint8_t fj = t == 13 ? fi : acc.flag(dx, dy, dz);
-    float nj[3] = {0.f, 0.f, 0.f}, aj = 0.f;
+    T nj[3] = {T(0), T(0), T(0)}, aj = T(0);
     const bool have = lane < 27 && ((fj & T_IF) || t == 13) && acc.normal(dx, dy, dz, nj, aj);
     const bool point = have && t != 13;
-    const float o[3] = {(float)dx, (float)dy, (float)dz};
-    const float dv[3] = {o[0] + aj * nj[0] - p[0], o[1] + aj * nj[1] - p[1], o[2] + aj * nj[2] - p[2]};
-    const float u = dot3(dv, tu), v = dot3(dv, tv), f = dot3(dv, n);
+    const T o[3] = {T((double)dx), T((double)dy), T((double)dz)};
+    const T dv[3] = {o[0] + aj * nj[0] - p[0], o[1] + aj * nj[1] - p[1], o[2] + aj * nj[2] - p[2]};
+    const T u = dot3(dv, tu), v = dot3(dv, tv), f = dot3(dv, n);
     bool touch = false;
-    float uj = 0.f, vj = 0.f, g1 = 0.f, g2 = 0.f;
+    T uj = T(0), vj = T(0), g1 = T(0), g2 = T(0);
     if (have && (fj & B_NEAR)) {
-        float pc[3], mh[3];
-        if (contact<float>(acc, dx, dy, dz, o, nj, aj, pc, mh)) {
-            const float mn = dot3(mh, n);
-            if (fabsf(mn) >= 1e-6f) {
-                const float dc[3] = {pc[0] - p[0], pc[1] - p[1], pc[2] - p[2]};
+        T pc[3], mh[3];
+        if (contact<T>(acc, dx, dy, dz, o, nj, aj, pc, mh)) {
+            const T mn = dot3(mh, n);
+            if (fabs(mn) >= T(1e-6)) {
+                const T dc[3] = {pc[0] - p[0], pc[1] - p[1], pc[2] - p[2]};
                 uj = dot3(dc, tu);
                 vj = dot3(dc, tv);
                 g1 = -dot3(mh, tu) / mn;
@@ -683,14 +688,14 @@ __device__ __forceinline__ float lsqr_warp(const Acc &acc, uint8_t fi, int lane,
     }
     // the centre's contact point constrains the gradient there
     const bool cons = __shfl_sync(all, touch ? 1 : 0, 13) != 0;
-    const float uc = __shfl_sync(all, uj, 13), vc = __shfl_sync(all, vj, 13);
-    const float gu = __shfl_sync(all, g1, 13), gv = __shfl_sync(all, g2, 13);
+    const T uc = __shfl_sync(all, uj, 13), vc = __shfl_sync(all, vj, 13);
+    const T gu = __shfl_sync(all, g1, 13), gv = __shfl_sync(all, g2, 13);
     const unsigned pm = __ballot_sync(all, point), tm = __ballot_sync(all, point && touch);
     const unsigned lt = (1u << lane) - 1u;
     const int m = __popc(pm) + 2 * __popc(tm);
     int at = __popc(pm & lt) + 2 * __popc(tm & lt);
-    auto put = [&](float a0, float a1, float a2, float a3, float a4, float r0, float r1, float r2, float b) {
-        float *q = rows.full[at], *r = rows.red[at];
+    auto put = [&](T a0, T a1, T a2, T a3, T a4, T r0, T r1, T r2, T b) {
+        T *q = rows.full[at], *r = rows.red[at];
         q[0] = a0; q[1] = a1; q[2] = a2; q[3] = a3; q[4] = a4; q[5] = b;
         r[0] = r0; r[1] = r1; r[2] = r2; r[3] = b;
         ++at;
@@ -699,15 +704,15 @@ __device__ __forceinline__ float lsqr_warp(const Acc &acc, uint8_t fi, int lane,
         if (!cons) {
             put(u * u, v * v, u * v, u, v, u * u + v * v, u, v, f);
             if (touch) {
-                put(2.f * uj, 0.f, vj, 1.f, 0.f, 2.f * uj, 1.f, 0.f, g1);
-                put(0.f, 2.f * vj, uj, 0.f, 1.f, 2.f * vj, 0.f, 1.f, g2);
+                put(T(2) * uj, T(0), vj, T(1), T(0), T(2) * uj, T(1), T(0), g1);
+                put(T(0), T(2) * vj, uj, T(0), T(1), T(2) * vj, T(0), T(1), g2);
             }
         } else {
-            put(u * u - 2.f * uc * u, v * v - 2.f * vc * v, u * v - vc * u - uc * v, 0.f, 0.f,
-                u * u + v * v - 2.f * uc * u - 2.f * vc * v, 0.f, 0.f, f - gu * u - gv * v);
+            put(u * u - T(2) * uc * u, v * v - T(2) * vc * v, u * v - vc * u - uc * v, T(0), T(0),
+                u * u + v * v - T(2) * uc * u - T(2) * vc * v, T(0), T(0), f - gu * u - gv * v);
             if (touch) {
-                put(2.f * (uj - uc), 0.f, vj - vc, 0.f, 0.f, 2.f * (uj - uc), 0.f, 0.f, g1 - gu);
-                put(0.f, 2.f * (vj - vc), uj - uc, 0.f, 0.f, 2.f * (vj - vc), 0.f, 0.f, g2 - gv);
+                put(T(2) * (uj - uc), T(0), vj - vc, T(0), T(0), T(2) * (uj - uc), T(0), T(0), g1 - gu);
+                put(T(0), T(2) * (vj - vc), uj - uc, T(0), T(0), T(2) * (vj - vc), T(0), T(0), g2 - gv);
             }
         }
     }
@@ -715,7 +720,7 @@ __device__ __forceinline__ float lsqr_warp(const Acc &acc, uint8_t fi, int lane,
     // pipelined Givens rotations
     const int j = lane & 7, kf = cons ? 3 : 5, kr = cons ? 1 : 3;
     const int cols = lane < 8 ? kf : (lane < 16 ? kr : 0);
-    float R[5] = {0.f, 0.f, 0.f, 0.f, 0.f}, qb = 0.f, w[5] = {0.f, 0.f, 0.f, 0.f, 0.f}, b = 0.f;
+    T R[5] = {T(0), T(0), T(0), T(0), T(0)}, qb = T(0), w[5] = {T(0), T(0), T(0), T(0), T(0)}, b = T(0);
     for (int it = 0; it < m + 4; ++it) {
         // the row: from shared memory for column 0, else what the column before made of it
 #pragma unroll
@@ -730,63 +735,78 @@ __device__ __forceinline__ float lsqr_warp(const Acc &acc, uint8_t fi, int lane,
             } else {
 #pragma unroll
                 for (int l = 0; l < 3; ++l) w[l] = rows.red[r][l];
-                w[3] = w[4] = 0.f;
+                w[3] = w[4] = T(0);
                 b = rows.red[r][3];
             }
         } else {
-            w[4] = 0.f;
+            w[4] = T(0);
         }
         if (j < cols && it >= j && it - j < m) {
-            const float h = sqrtf(R[0] * R[0] + w[0] * w[0]);
-            if (h != 0.f) {
-                const float c = R[0] / h, s = w[0] / h;
+            const T h = sqrt(R[0] * R[0] + w[0] * w[0]);
+            if (h != T(0)) {
+                const T c = R[0] / h, s = w[0] / h;
                 R[0] = h;
 #pragma unroll
                 for (int l = 1; l < 5; ++l) {
-                    const float r = R[l];
+                    const T r = R[l];
                     R[l] = c * r + s * w[l];
                     w[l] = c * w[l] - s * r;
                 }
-                const float z = qb;
+                const T z = qb;
                 qb = c * z + s * b;
                 b = c * b - s * z;
             }
         }
     }
-    Givens<float, 5> full;
-    Givens<float, 3> red;
+    Givens<T, 5> full;
+    Givens<T, 3> red;
 #pragma unroll
     for (int r = 0; r < 5; ++r) {
 #pragma unroll
-        for (int c = r; c < 5; ++c) full.R[Givens<float, 5>::at(r, c)] = __shfl_sync(all, R[c - r], r);
+        for (int c = r; c < 5; ++c) full.R[Givens<T, 5>::at(r, c)] = __shfl_sync(all, R[c - r], r);
         full.qb[r] = __shfl_sync(all, qb, r);
     }
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
 #pragma unroll
-        for (int c = r; c < 3; ++c) red.R[Givens<float, 3>::at(r, c)] = __shfl_sync(all, R[c - r], 8 + r);
+        for (int c = r; c < 3; ++c) red.R[Givens<T, 3>::at(r, c)] = __shfl_sync(all, R[c - r], 8 + r);
         red.qb[r] = __shfl_sync(all, qb, 8 + r);
     }
     __syncwarp();
-    float A, B, C, H, I, sol[5] = {0.f, 0.f, 0.f, 0.f, 0.f}, c2;
+    T A, B, C, H, I, sol[5] = {T(0), T(0), T(0), T(0), T(0)}, c2;
     if (m >= kf && full.solve(sol, kf, c2)) {
         A = sol[0];
         B = sol[1];
         C = sol[2];
-        H = cons ? gu - 2.f * uc * A - vc * C : sol[3];
-        I = cons ? gv - 2.f * vc * B - uc * C : sol[4];
+        H = cons ? gu - T(2) * uc * A - vc * C : sol[3];
+        I = cons ? gv - T(2) * vc * B - uc * C : sol[4];
     } else {
-        float xr[3] = {0.f, 0.f, 0.f};
+        T xr[3] = {T(0), T(0), T(0)};
         if (m >= kf) cond = c2;  // the full model's, as lsqr_core reports a fit it could not take
-        if (!(m >= kr && red.solve(xr, kr, c2))) return 0.f;
+        if (!(m >= kr && red.solve(xr, kr, c2))) return T(0);
         A = B = xr[0];
-        C = 0.f;
-        H = cons ? gu - 2.f * uc * A : xr[1];
-        I = cons ? gv - 2.f * vc * A : xr[2];
+        C = T(0);
+        H = cons ? gu - T(2) * uc * A : xr[1];
+        I = cons ? gv - T(2) * vc * A : xr[2];
     }
     cond = c2;
-    const float g = 1.f + H * H + I * I;
-    return (A * (1.f + I * I) + B * (1.f + H * H) - C * H * I) / (g * sqrtf(g));
+    const T g = T(1) + H * H + I * I;
+    return (A * (T(1) + I * I) + B * (T(1) + H * H) - C * H * I) / (g * sqrt(g));
+}
+
+// The general fit by a warp, re-solved in FP64 (the same pipeline) where the
+// FP32 factor is ill conditioned: necks of merging droplets have many such cells,
+// and one lane took about 100 us for a fit in FP64.
+template <typename Acc>
+__device__ __forceinline__ float general_fit_warp(const Dev &d, const Acc &acc, uint8_t fi, int lane, FitRows &rows) {
+    float cond;
+    float kap = lsqr_warp<float>(acc, fi, lane, rows.f, cond);
+    if (cond * cond > d.fp64_cond) {  // warp-uniform
+        double c2;
+        kap = (float)lsqr_warp<double>(acc, fi, lane, rows.d, c2);
+        if (lane == 0) atomicAdd(d.counts + C_FP64, 1);
+    }
+    return kap;
 }
 
 // Fast path: FP32 normal equations of the full model for an interface cell

@@ -124,9 +124,8 @@ __global__ void __launch_bounds__(LIST_THREADS) k_lsqr_slow(const __grid_constan
         __syncwarp();
         const StagedAcc acc{d, sfl[w], snm[w]};
         const uint8_t fi = d.flags[i];
-        float cond;
-        const float kap = lsqr_warp(acc, fi, lane, rows[w], cond);
-        if (lane == 0) kappa_out[i] = cond * cond > d.fp64_cond ? general_fit_fp64(d, acc, fi) : kap;
+        const float kap = general_fit_warp(d, acc, fi, lane, rows[w]);
+        if (lane == 0) kappa_out[i] = kap;
         __syncwarp();
     }
 }

@@ -84,8 +84,7 @@ __global__ void __launch_bounds__(LIST_BLOCK, IFACE_MIN_BLOCKS) k_curv_iface_fas
 
 // General-path cells (contact-line cells, degenerate or ill-conditioned FP32
 // fits): one warp per cell stages the block in shared memory and runs the
-// Givens fit as a pipeline over its lanes (lsqr_warp; FP64 by one lane when
-// ill conditioned), then one lane the interface stream-collide of the cell.
+// Givens fit as a pipeline over its lanes (general_fit_warp), then one lane the interface stream-collide of the cell.
 // PIPE: the fit by lsqr_warp; else lsqr_core by one lane.  The two differ in
 // which products are fused (kappa by about 1e-7), and a window's gradients
 // magnify the last bits of its states near full and empty cells, so the frozen
@@ -110,10 +109,8 @@ __global__ void __launch_bounds__(LIST_BLOCK) k_curv_iface_slow(const __grid_con
         const StagedAcc acc{d, sfl[w], snm[w]};
         if (PIPE) {
             const uint8_t fi = d.flags[i] & (T_MASK | B_NEAR);
-            float cond;
-            float kap = lsqr_warp(acc, fi, lane, rows[w], cond);
+            const float kap = general_fit_warp(d, acc, fi, lane, rows[w]);
             if (lane == 0) {
-                if (cond * cond > d.fp64_cond) kap = general_fit_fp64(d, acc, fi);
                 d.kappa[i] = kap;
                 iface_cell<S, COLL>(d, i);
             }
