@@ -387,6 +387,12 @@ def launches_per_step(curv, obs):
     return 7
 
 
+def kernels_per_step(curv, obs):
+    """The same less the normals, which FD curvature leaves out in a domain
+    without obstacles."""
+    return launches_per_step(curv, obs) - (1 if curv == "fd" and (obs is None or not bool(obs.any())) else 0)
+
+
 def measured_traffic(kernel, workload):
     """DRAM bytes per launch from the committed ncu capture (profiles/ncu_traffic.json),
     or None when the kernel's source changed since the capture."""
@@ -1106,7 +1112,7 @@ def run_fsl(args):
             "lsqr_fp64_cells": n_fp64,
             "phases_ms": dict(zip(PHASES, [round(float(v), 5) for v in ph])),
             "mass_reduce_ms": mass_ms, "mass_drift_rel": drift, "roofline": roof, "e2e": e2e,
-            "gpu_launches": launches_per_step(args.curv, obs) * args.steps, "clocks": clocks}
+            "gpu_launches": kernels_per_step(args.curv, obs) * args.steps, "clocks": clocks}
     gs = None
     if rank == 0 and ws == 1 and not args.no_cpu_baseline:
         gs = {"flags": sim2.flags_current().cpu().numpy(), "phi": sim2.phi.double().cpu().numpy()}

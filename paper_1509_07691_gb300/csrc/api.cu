@@ -24,7 +24,7 @@ struct fsl_ctx {
     cudaEvent_t fork, join;
     int parity;
     Dev base;                // pointers and parameters common to both parities
-    cudaGraphExec_t graph[2];
+    cudaGraphExec_t graph[4];  // one step from parity 0, 1; two steps from parity 0, 1
     double *mass_out;        // 2 doubles in the workspace
     double *host_mass;       // pinned, 4 doubles (mass, lost; dL/dsigma, dL/dtheta)
     long long *host_stats;   // pinned
@@ -192,7 +192,7 @@ int read_near(fsl_ctx *c) {
     CK(cudaStreamSynchronize(c->stream));
     const int inl = *c->host_count == 0 ? 1 : 0;
     if (inl != c->base.inline_general)
-        for (int k = 0; k < 2; ++k)
+        for (int k = 0; k < 4; ++k)
             if (c->graph[k]) {
                 cudaGraphExecDestroy(c->graph[k]);
                 c->graph[k] = nullptr;
@@ -241,13 +241,15 @@ int enqueue_step_graph(const fsl_ctx *c, int parity) {
     return cudaGetLastError() == cudaSuccess ? FSL_OK : FSL_ECUDA;
 }
 
-int record_graph(fsl_ctx *c, int parity) {
+// graph of `steps` (1 or 2) steps from the given parity
+int record_graph(fsl_ctx *c, int parity, int steps) {
     cudaGraph_t g;
     CK(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
-    const int rc = enqueue_step_graph(c, parity);
+    int rc = FSL_OK;
+    for (int k = 0; k < steps && rc == FSL_OK; ++k) rc = enqueue_step_graph(c, parity ^ k);
     cudaError_t e = cudaStreamEndCapture(c->cap_stream, &g);
     if (rc != FSL_OK || e != cudaSuccess) return FSL_ECUDA;
-    e = cudaGraphInstantiate(&c->graph[parity], g, 0);
+    e = cudaGraphInstantiate(&c->graph[2 * (steps - 1) + parity], g, 0);
     cudaGraphDestroy(g);
     return e == cudaSuccess ? FSL_OK : FSL_ECUDA;
 }
@@ -492,13 +494,18 @@ int fsl_step(fsl_ctx *c, int nsteps) {
     if (!c || nsteps < 0) return FSL_EINVAL;
     if (nsteps > 0) c->adj_valid = 0;
     if (c->p.curv_model == FSL_CURV_MLP && !c->base.mlp_params) return FSL_EINVAL;
-    for (int s = 0; s < nsteps; ++s) {
-        if (!c->graph[c->parity]) {
-            const int rc = record_graph(c, c->parity);
+    // steps in pairs, which return to the same parity: one graph instead of two
+    // to record and half the launches, and the second step's first kernel is
+    // dispatched while the first step drains
+    for (int s = 0; s < nsteps;) {
+        const int steps = nsteps - s >= 2 ? 2 : 1, k = 2 * (steps - 1) + c->parity;
+        if (!c->graph[k]) {
+            const int rc = record_graph(c, c->parity, steps);
             if (rc != FSL_OK) return rc;
         }
-        CK(cudaGraphLaunch(c->graph[c->parity], c->stream));
-        c->parity ^= 1;
+        CK(cudaGraphLaunch(c->graph[k], c->stream));
+        c->parity ^= steps & 1;
+        s += steps;
     }
     return FSL_OK;
 }
@@ -565,7 +572,7 @@ int fsl_mlp_attach(fsl_ctx *c, const void *params, double fallback_rel) {
     c->base.mlp_params = static_cast<const uint8_t *>(params);
     c->base.mlp_rel = (float)fallback_rel;
     // recorded graphs hold the old parameters
-    for (int k = 0; k < 2; ++k)
+    for (int k = 0; k < 4; ++k)
         if (c->graph[k]) {
             cudaGraphExecDestroy(c->graph[k]);
             c->graph[k] = nullptr;
@@ -602,7 +609,7 @@ static int bubble_volume(fsl_ctx *c, double *V) {
 
 int fsl_set_bubble(fsl_ctx *c, double p0, double V0) {
     if (!c || !isfinite(p0) || !isfinite(V0) || p0 < 0.0) return FSL_EINVAL;
-    for (int k = 0; k < 2; ++k)  // recorded graphs hold the old kernel arguments
+    for (int k = 0; k < 4; ++k)  // recorded graphs hold the old kernel arguments
         if (c->graph[k]) {
             cudaGraphExecDestroy(c->graph[k]);
             c->graph[k] = nullptr;
@@ -709,7 +716,7 @@ int fsl_set_surface(fsl_ctx *c, double sigma, double theta) {
     c->base.sin_theta = (float)sin(theta);
     c->base.cos_theta_d = cos(theta);
     c->base.sin_theta_d = sin(theta);
-    for (int k = 0; k < 2; ++k)
+    for (int k = 0; k < 4; ++k)
         if (c->graph[k]) {
             cudaGraphExecDestroy(c->graph[k]);
             c->graph[k] = nullptr;
@@ -961,7 +968,7 @@ const char *fsl_strerror(int code) {
 
 void fsl_destroy(fsl_ctx *c) {
     if (!c) return;
-    for (int k = 0; k < 2; ++k)
+    for (int k = 0; k < 4; ++k)
         if (c->graph[k]) cudaGraphExecDestroy(c->graph[k]);
     if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
     if (c->cap_side) cudaStreamDestroy(c->cap_side);

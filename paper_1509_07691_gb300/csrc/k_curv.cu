@@ -435,7 +435,7 @@ __global__ void k_zero_kappa(Dev d, float *kappa_out) {
 
 void launch_normals(const Dev &d, cudaStream_t s) {
     static const int g = list_blocks((const void *)k_normals, LIST_THREADS, 4);
-    k_normals<<<g, LIST_THREADS, 0, s>>>(d);
+    launch_pdl(k_normals, g, LIST_THREADS, s, d);
 }
 void launch_lsqr(const Dev &d, float *kappa_out, cudaStream_t s) {
     static const int gf = list_blocks((const void *)k_lsqr_fast, LIST_THREADS, 4);

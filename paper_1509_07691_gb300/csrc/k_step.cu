@@ -48,8 +48,10 @@ __global__ void __launch_bounds__(LIST_BLOCK) k_sc_iface(Dev d) {
 // cell; k_curv_iface_slow finishes the deferred cells one thread each (Givens
 // fit, FP64 re-solve when ill conditioned, then iface_cell).  In a domain
 // without obstacles (no contact lines: a deferral is a rare ill-conditioned
-// or degenerate fit) the fused kernel's last block finishes the deferred
-// cells and k_curv_iface_slow is not launched.
+// or degenerate fit) a step leaves them to k_convert, and k_curv_iface_slow is
+// not launched.  (The fused kernel's last block finished them before; the fence
+// by which that block was found held every block until its stores had landed,
+// 2 us a step.)
 // iface_cell of one cell changes only that cell's transient flag bits, mass,
 // rho and new PDFs, none of which a fit of another cell reads.
 constexpr int IFACE_MIN_BLOCKS = 3;
@@ -64,22 +66,6 @@ __global__ void __launch_bounds__(LIST_BLOCK, IFACE_MIN_BLOCKS) k_curv_iface_fas
     const int lane = threadIdx.x & 31;
     const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), nwarps = (int)((gridDim.x * blockDim.x) >> 5);
     for (int base = gw * CPW; base < n; base += nwarps * CPW) curv_iface_task<S, COLL, L>(d, base, n, lane);
-    // without obstacles the last block to finish runs the deferred fits (rare
-    // ill-conditioned or degenerate ones), one thread per cell: every block's
-    // list appends are fenced before its arrival is counted
-    if (d.inline_general) {  // uniform over the grid
-        __shared__ int last;
-        __threadfence();
-        __syncthreads();
-        if (threadIdx.x == 0) last = atomicAdd(d.counts + C_IFDONE, 1) == (int)gridDim.x - 1;
-        __syncthreads();
-        if (last) {
-            __threadfence();
-            const int ns = __ldcg(d.counts + C_SLOW);
-            for (int k = threadIdx.x; k < ns; k += blockDim.x) general_cell_grid<S, COLL>(d, __ldcg(d.slow + k));
-            if (threadIdx.x == 0) d.counts[C_IFDONE] = 0;
-        }
-    }
 }
 
 // General-path cells (contact-line cells, degenerate or ill-conditioned FP32
@@ -126,10 +112,18 @@ __global__ void __launch_bounds__(LIST_BLOCK) k_curv_iface_slow(const __grid_con
 // converts few cells, and one block keeps every phase visible to the next.
 constexpr int CONV_BLOCK = 1024;
 
-template <int S>
-__global__ void __launch_bounds__(CONV_BLOCK) k_convert(Dev d) {
+template <int S, int COLL>
+__global__ void __launch_bounds__(CONV_BLOCK) k_convert(const __grid_constant__ Dev d) {
     pdl_enter();
-    const int nfill = __ldcg(d.counts + C_FILL), nempty = __ldcg(d.counts + C_EMPTY);
+    int nfill = __ldcg(d.counts + C_FILL), nempty = __ldcg(d.counts + C_EMPTY);
+    const int nslow = __ldcg(d.counts + C_SLOW);
+    // without obstacles: the fits the fused kernel deferred, one thread per cell
+    if (nslow && d.inline_general && d.curv_model == FSL_CURV_LSQR) {
+        for (int k = threadIdx.x; k < nslow; k += blockDim.x) general_cell_grid<S, COLL>(d, d.slow[k]);
+        __syncthreads();
+        nfill = __ldcg(d.counts + C_FILL);
+        nempty = __ldcg(d.counts + C_EMPTY);
+    }
     if (nfill + nempty == 0) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     for (int k = warp; k < nfill + nempty; k += nwarps) convert_mark(d, k, nfill, lane);
@@ -247,12 +241,18 @@ void launch_ci(const Dev &d, cudaStream_t s) {
     static const int gs = list_blocks((const void *)k_curv_iface_slow<S, COLL, true>, LIST_BLOCK, 4);
     static const int gz = list_blocks((const void *)k_curv_iface_slow<S, COLL, false>, LIST_BLOCK, 4);
     launch_pdl(k_curv_iface_fast<S, COLL, FSL_IFACE_LANES>, gf, LIST_BLOCK, s, d);
-    if (d.inline_general) return;
+    if (d.inline_general && !d.frozen) return;  // k_convert finishes the few deferred fits
     if (d.frozen) launch_pdl(k_curv_iface_slow<S, COLL, false>, gz, LIST_BLOCK, s, d);
     else launch_pdl(k_curv_iface_slow<S, COLL, true>, gs, LIST_BLOCK, s, d);
 }
 
+template <int S, int COLL>
+void launch_conv(const Dev &d, cudaStream_t s) {
+    launch_pdl(k_convert<S, COLL>, 1, CONV_BLOCK, s, d);
+}
+
 void launch_sc_bulk(const Dev &d, cudaStream_t s) { FSL_DISPATCH(launch_bulk); }
+void launch_convert(const Dev &d, cudaStream_t s) { FSL_DISPATCH(launch_conv); }
 void launch_curv_iface(const Dev &d, cudaStream_t s) { FSL_DISPATCH(launch_ci); }
 void launch_sc_iface(const Dev &d, cudaStream_t s) { FSL_DISPATCH(launch_iface); }
 #undef FSL_DISPATCH
@@ -260,14 +260,6 @@ void launch_sc_iface(const Dev &d, cudaStream_t s) { FSL_DISPATCH(launch_iface);
 void launch_stream_collide(const Dev &d, cudaStream_t s) {
     launch_sc_bulk(d, s);
     launch_sc_iface(d, s);
-}
-
-void launch_convert(const Dev &d, cudaStream_t s) {
-    switch (d.storage) {
-    case FSL_F32: launch_pdl(k_convert<FSL_F32>, 1, CONV_BLOCK, s, d); break;
-    case FSL_F16_OFS: launch_pdl(k_convert<FSL_F16_OFS>, 1, CONV_BLOCK, s, d); break;
-    default: launch_pdl(k_convert<FSL_BF16_OFS>, 1, CONV_BLOCK, s, d); break;
-    }
 }
 
 void launch_finalize(const Dev &d, cudaStream_t s) {

@@ -200,12 +200,12 @@ __device__ __forceinline__ void general_cell(const Dev &d, const Acc &acc, int i
     iface_cell<S, COLL>(d, i);
 }
 
-// the same, by one thread reading the block from global memory: the fused
-// kernel's own deferred cells in a domain without obstacles (no contact
-// lines, so deferrals are rare ill-conditioned fits); out of line, so that the
-// fused kernel's registers are not spent on it
+// the same, by one thread reading the block from global memory: a deferred cell
+// in a domain without obstacles (no contact lines, so deferrals are rare
+// ill-conditioned fits); out of line, so that k_convert's registers are not
+// spent on it
 template <int S, int COLL>
-__device__ __noinline__ void general_cell_grid(const Dev d, int i) {
+__device__ __noinline__ void general_cell_grid(const Dev &d, int i) {
     int x, y, z;
     cell_coords(d, i, x, y, z);
     const GridAcc acc{d, x, y, z};
