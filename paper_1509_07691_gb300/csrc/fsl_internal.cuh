@@ -210,7 +210,7 @@ template <>
 struct Store<FSL_F32> {
     using T = float;
     __device__ static __forceinline__ float ld(const void *p, long long k, int q, const Dev &) {
-        return static_cast<const float *>(p)[k];
+        return __ldg(static_cast<const float *>(p) + k);
     }
     __device__ static __forceinline__ float ldcg(const void *p, long long k, int q, const Dev &) {
         return __ldcg(static_cast<const float *>(p) + k);
@@ -222,7 +222,7 @@ struct Store<FSL_F32> {
     __device__ static __forceinline__ void put(float &o, float v, float w, const Dev &) { o = v; }
     // direction q of cell i
     __device__ static __forceinline__ float ld_at(const void *p, int q, unsigned i, const Dev &d) {
-        return (static_cast<const float *>(p) + (long long)q * d.N)[i];
+        return __ldg(static_cast<const float *>(p) + (long long)q * d.N + i);
     }
     __device__ static __forceinline__ void st_at(void *p, int q, unsigned i, float v, const Dev &d) {
         (static_cast<float *>(p) + (long long)q * d.N)[i] = v;
@@ -232,7 +232,7 @@ template <>
 struct Store<FSL_F16_OFS> {
     using T = __half;
     __device__ static __forceinline__ float ld(const void *p, long long k, int q, const Dev &d) {
-        return fmaf(__half2float(static_cast<const __half *>(p)[k]), d.inv_scale, wq(q));
+        return fmaf(__half2float(__ldg(static_cast<const __half *>(p) + k)), d.inv_scale, wq(q));
     }
     __device__ static __forceinline__ float ldcg(const void *p, long long k, int q, const Dev &d) {
         return fmaf(__half2float(__ldcg(static_cast<const __half *>(p) + k)), d.inv_scale, wq(q));
@@ -242,7 +242,7 @@ struct Store<FSL_F16_OFS> {
     }
     __device__ static __forceinline__ void put(__half &o, float v, float w, const Dev &d) { o = __float2half_rn((v - w) * d.scale); }
     __device__ static __forceinline__ float ld_at(const void *p, int q, unsigned i, const Dev &d) {
-        const __half h = (static_cast<const __half *>(p) + (long long)q * d.N)[i];
+        const __half h = __ldg(static_cast<const __half *>(p) + (long long)q * d.N + i);
         return fmaf(__half2float(h), d.inv_scale, wq(q));
     }
     __device__ static __forceinline__ void st_at(void *p, int q, unsigned i, float v, const Dev &d) {
@@ -253,7 +253,7 @@ template <>
 struct Store<FSL_BF16_OFS> {
     using T = __nv_bfloat16;
     __device__ static __forceinline__ float ld(const void *p, long long k, int q, const Dev &d) {
-        return fmaf(__bfloat162float(static_cast<const __nv_bfloat16 *>(p)[k]), d.inv_scale, wq(q));
+        return fmaf(__bfloat162float(__ldg(static_cast<const __nv_bfloat16 *>(p) + k)), d.inv_scale, wq(q));
     }
     __device__ static __forceinline__ float ldcg(const void *p, long long k, int q, const Dev &d) {
         return fmaf(__bfloat162float(__ldcg(static_cast<const __nv_bfloat16 *>(p) + k)), d.inv_scale, wq(q));
@@ -263,7 +263,7 @@ struct Store<FSL_BF16_OFS> {
     }
     __device__ static __forceinline__ void put(__nv_bfloat16 &o, float v, float w, const Dev &d) { o = __float2bfloat16_rn((v - w) * d.scale); }
     __device__ static __forceinline__ float ld_at(const void *p, int q, unsigned i, const Dev &d) {
-        const __nv_bfloat16 h = (static_cast<const __nv_bfloat16 *>(p) + (long long)q * d.N)[i];
+        const __nv_bfloat16 h = __ldg(static_cast<const __nv_bfloat16 *>(p) + (long long)q * d.N + i);
         return fmaf(__bfloat162float(h), d.inv_scale, wq(q));
     }
     __device__ static __forceinline__ void st_at(void *p, int q, unsigned i, float v, const Dev &d) {

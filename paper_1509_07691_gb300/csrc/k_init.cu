@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(256) k_init_state(Dev d, const uint8_t *tmp, i
         uint8_t t = tmp[i];
         bool gas_nbr = false;
         // only a liquid cell, or any cell of a domain with obstacles, depends on its
-        // neighbours: most cells of a droplet's box are gas (170 us on 256^3 with every cell looking, 85 now)
+        // neighbours: most cells of a droplet's box are gas (170 us on 256^3 with every cell looking, 81 now)
         if (walls || t == T_LIQ) {
             for (int q = 1; q < Q; ++q) {
                 const uint8_t u = tmp[nbr_index(d, x, y, z, cx(q), cy(q), cz(q))];

@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(LIST_BLOCK) k_sc_iface(Dev d) {
 // one pass: k_curv_iface_fast fits the cell by the FP32 normal equations
 // (as k_lsqr_fast) and, unless the fit defers the cell to the general path,
 // goes straight on with the cell's stream-collide, FSL_IFACE_LANES lanes per
-// cell; k_curv_iface_slow finishes the deferred cells one thread each (Givens
+// cell; k_curv_iface_slow finishes the deferred cells one warp each (Givens
 // fit, FP64 re-solve when ill conditioned, then iface_cell).  In a domain
 // without obstacles (no contact lines: a deferral is a rare ill-conditioned
 // or degenerate fit) a step leaves them to k_convert, and k_curv_iface_slow is
