@@ -141,23 +141,9 @@ __device__ S plic_alpha(S m1, S m2, S m3, S phi, int iters) {
 }
 
 // Offset a of the plane {y.n = a} through the cell [-1/2,1/2]^3 whose liquid
-// side {y.n >= a} holds volume phi.  With m = |n| / sum|n| and
-// al = 1/2 - a / sum|n| the liquid part is {z : m.z <= al} of the unit cube.
-template <typename S>
-__device__ S plic_offset(S nx, S ny, S nz, S phi, int iters) {
-    S a1 = fabs(nx), a2 = fabs(ny), a3 = fabs(nz);
-    const S M = a1 + a2 + a3;
-    if (phi <= S(0)) return 0.5f * M;
-    if (phi >= S(1)) return -0.5f * M;
-    S t;
-    if (a1 > a2) { t = a1; a1 = a2; a2 = t; }
-    if (a2 > a3) { t = a2; a2 = a3; a3 = t; }
-    if (a1 > a2) { t = a1; a1 = a2; a2 = t; }
-    const S m1 = a1 / M, m2 = a2 / M, m3 = S(1) - m1 - m2;
-    return M * (0.5f - plic_alpha(m1, m2, m3, phi, iters));
-}
-
-// The same offset for dual inputs: the value by plic_offset's arithmetic, the
+// side {y.n >= a} holds volume phi, for dual inputs (plain ones: plic_normal_rn).
+// With m = |n| / sum|n| and al = 1/2 - a / sum|n| the liquid part is
+// {z : m.z <= al} of the unit cube; the value by plic_alpha, the
 // derivative by the implicit function theorem on V(al; m) = phi,
 // dal = (dphi - dV/dm . dm) / (dV/dal), exact at the computed al.
 template <typename S>
