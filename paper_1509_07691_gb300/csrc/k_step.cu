@@ -46,18 +46,22 @@ __global__ void __launch_bounds__(LIST_BLOCK) k_sc_iface(Dev d) {
 // (as k_lsqr_fast) and, unless the fit defers the cell to the general path,
 // goes straight on with the cell's stream-collide, FSL_IFACE_LANES lanes per
 // cell; k_curv_iface_slow finishes the deferred cells one warp each (Givens
-// fit, FP64 re-solve when ill conditioned, then iface_cell).  In a domain
-// without obstacles (no contact lines: a deferral is a rare ill-conditioned
-// or degenerate fit) a step leaves them to k_convert, and k_curv_iface_slow is
-// not launched.  (The fused kernel's last block finished them before; the fence
-// by which that block was found held every block until its stores had landed,
-// 2 us a step.)
+// fit, FP64 re-solve when ill conditioned, then iface_cell).  In a step of a
+// domain without obstacles (no contact lines: a deferral is an ill-conditioned
+// or degenerate fit) each warp finishes its own after its share of the list, one
+// lane each, and k_curv_iface_slow is not launched: a serial fit then costs its
+// own warp only, and many of them (necks of merging droplets, a low
+// lsqr_fp64_cond) spread over the GPU.  Ten steps of two touching droplets in
+// 128^3: 1.10 ms; 1.49 with the fits in this kernel's last block behind a fence,
+// 1.60 in the conversion kernel (one block behind the liquid pass, 64 registers
+// a thread), 1.11 with k_curv_iface_slow launched in every step, which costs 2.5 us
+// a step where nothing is deferred (32^3 droplet, ten steps: 225, 276, 232 and 256 us).
 // iface_cell of one cell changes only that cell's transient flag bits, mass,
 // rho and new PDFs, none of which a fit of another cell reads.
 constexpr int IFACE_MIN_BLOCKS = 3;
 
 template <int S, int COLL, int L>
-__global__ void __launch_bounds__(LIST_BLOCK, IFACE_MIN_BLOCKS) k_curv_iface_fast(Dev d) {
+__global__ void __launch_bounds__(LIST_BLOCK, IFACE_MIN_BLOCKS) k_curv_iface_fast(const __grid_constant__ Dev d) {
     pdl_enter();
     int cnt[1];
     block_counts<1>(d.counts, {d.cif}, cnt);
@@ -65,7 +69,11 @@ __global__ void __launch_bounds__(LIST_BLOCK, IFACE_MIN_BLOCKS) k_curv_iface_fas
     constexpr int CPW = 32 / L;  // cells per warp
     const int lane = threadIdx.x & 31;
     const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), nwarps = (int)((gridDim.x * blockDim.x) >> 5);
-    for (int base = gw * CPW; base < n; base += nwarps * CPW) curv_iface_task<S, COLL, L>(d, base, n, lane);
+    int later = 0;  // this warp's deferred cells (steps without obstacles)
+    for (int base = gw * CPW; base < n; base += nwarps * CPW)
+        curv_iface_task<S, COLL, L>(d, base, n, lane, gw, nwarps * CPW, later);
+    __syncwarp();
+    for (int j = lane; j < later; j += 32) general_cell_grid<S, COLL>(d, d.slow[own_place(gw, CPW, nwarps * CPW, j)]);
 }
 
 // General-path cells (contact-line cells, degenerate or ill-conditioned FP32
@@ -112,18 +120,10 @@ __global__ void __launch_bounds__(LIST_BLOCK) k_curv_iface_slow(const __grid_con
 // converts few cells, and one block keeps every phase visible to the next.
 constexpr int CONV_BLOCK = 1024;
 
-template <int S, int COLL>
-__global__ void __launch_bounds__(CONV_BLOCK) k_convert(const __grid_constant__ Dev d) {
+template <int S>
+__global__ void __launch_bounds__(CONV_BLOCK) k_convert(Dev d) {
     pdl_enter();
-    int nfill = __ldcg(d.counts + C_FILL), nempty = __ldcg(d.counts + C_EMPTY);
-    const int nslow = __ldcg(d.counts + C_SLOW);
-    // without obstacles: the fits the fused kernel deferred, one thread per cell
-    if (nslow && d.inline_general && d.curv_model == FSL_CURV_LSQR) {
-        for (int k = threadIdx.x; k < nslow; k += blockDim.x) general_cell_grid<S, COLL>(d, d.slow[k]);
-        __syncthreads();
-        nfill = __ldcg(d.counts + C_FILL);
-        nempty = __ldcg(d.counts + C_EMPTY);
-    }
+    const int nfill = __ldcg(d.counts + C_FILL), nempty = __ldcg(d.counts + C_EMPTY);
     if (nfill + nempty == 0) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     for (int k = warp; k < nfill + nempty; k += nwarps) convert_mark(d, k, nfill, lane);
@@ -241,14 +241,14 @@ void launch_ci(const Dev &d, cudaStream_t s) {
     static const int gs = list_blocks((const void *)k_curv_iface_slow<S, COLL, true>, LIST_BLOCK, 4);
     static const int gz = list_blocks((const void *)k_curv_iface_slow<S, COLL, false>, LIST_BLOCK, 4);
     launch_pdl(k_curv_iface_fast<S, COLL, FSL_IFACE_LANES>, gf, LIST_BLOCK, s, d);
-    if (d.inline_general && !d.frozen) return;  // k_convert finishes the few deferred fits
+    if (d.inline_general && !d.frozen) return;  // the fused kernel finished its deferred fits itself
     if (d.frozen) launch_pdl(k_curv_iface_slow<S, COLL, false>, gz, LIST_BLOCK, s, d);
     else launch_pdl(k_curv_iface_slow<S, COLL, true>, gs, LIST_BLOCK, s, d);
 }
 
 template <int S, int COLL>
 void launch_conv(const Dev &d, cudaStream_t s) {
-    launch_pdl(k_convert<S, COLL>, 1, CONV_BLOCK, s, d);
+    launch_pdl(k_convert<S>, 1, CONV_BLOCK, s, d);
 }
 
 void launch_sc_bulk(const Dev &d, cudaStream_t s) { FSL_DISPATCH(launch_bulk); }

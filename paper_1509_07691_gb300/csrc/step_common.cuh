@@ -200,9 +200,10 @@ __device__ __forceinline__ void general_cell(const Dev &d, const Acc &acc, int i
     iface_cell<S, COLL>(d, i);
 }
 
-// the same, by one thread reading the block from global memory: a deferred cell
-// in a domain without obstacles (no contact lines, so deferrals are rare
-// ill-conditioned fits); out of line, so that k_convert's registers are not
+// the same, by one thread reading the block from global memory: a cell the fast
+// fit deferred in a step of a domain without obstacles (no contact lines: an
+// ill-conditioned or degenerate fit, a few per step and more of them in the necks
+// of merging droplets); out of line, so that the fused kernel's registers are not
 // spent on it
 template <int S, int COLL>
 __device__ __noinline__ void general_cell_grid(const Dev &d, int i) {
@@ -234,11 +235,20 @@ __device__ __forceinline__ int group_or(int v) {
 #ifndef FSL_IFACE_LANES
 #define FSL_IFACE_LANES 2
 #endif
+// list position of the j-th cell of warp gw, which takes `cells` consecutive ones of
+// every `stride`
+__device__ __forceinline__ int own_place(int gw, int cells, int stride, int j) {
+    return gw * cells + j / cells * stride + j % cells;
+}
+
 // LSQR fit and interface stream-collide of the list cells base .. base + 32/L - 1
-// by one warp, L lanes per cell (see k_curv_iface_fast); cells whose fit needs
-// the general path go to d.slow.  The whole warp must call it.
+// by one warp, L lanes per cell (see k_curv_iface_fast).  A cell whose fit needs
+// the general path is left to k_curv_iface_slow (list d.slow), in a step without
+// obstacles to this warp itself: its later-th such cell is noted in d.slow at the
+// place of the later-th list cell the warp has visited (see own_place), so that no
+// other warp or counter is involved.  The whole warp must call it.
 template <int S, int COLL, int L>
-__device__ __forceinline__ void curv_iface_task(const Dev &d, int base, int n, int lane) {
+__device__ __forceinline__ void curv_iface_task(const Dev &d, int base, int n, int lane, int gw, int stride, int &later) {
     using St = Store<S>;
     const long long N = d.N;
     constexpr int RS = (27 + L - 1) / L;  // fit rows per lane
@@ -428,7 +438,13 @@ __device__ __forceinline__ void curv_iface_task(const Dev &d, int base, int n, i
         }
     }
     if (act && r == L - 1) St::st(d.fdst, i, 0, fo0 + d.omega_e * ((1.0f / 3.0f) * rg * (1.0f - vv) - fo0), d);
-    warp_append(d.slow, d.counts + C_SLOW, defer && r == 0, i);
+    if (d.inline_general && !d.frozen) {
+        const unsigned dm = __ballot_sync(0xffffffffu, defer && r == 0);
+        if (defer && r == 0) d.slow[own_place(gw, 32 / L, stride, later + __popc(dm & ((1u << lane) - 1u)))] = i;
+        later += __popc(dm);
+    } else {
+        warp_append(d.slow, d.counts + C_SLOW, defer && r == 0, i);
+    }
     if (act && r == 0) {
         d.kappa[i] = kap;
         const float mm = d.mass[i] + dm;
