@@ -306,8 +306,10 @@ int fsl_mlp_master_count(void);
  * levels by sub^3 sub-sampling, Gaussian noise of s.d. `noise` on partially
  * filled cells (splitmix64 at counters 2k, 2k+1 for stencil cell k of sample s,
  * k = 125 s + cell, Box-Muller; clipped to [0, 1]), written as canonical BF16
- * rows X [n][128], and the target: mean curvature at the surface point nearest
- * the middle cell's centre (negative for liquid outside).  Asynchronous. */
+ * rows X [n][128] (any address of a BF16 value; FSL_EINVAL for an odd one, and
+ * note that the network calls want X on a 16-byte boundary), and the target: mean
+ * curvature at the surface point nearest the middle cell's centre (negative for
+ * liquid outside).  Asynchronous. */
 int fsl_mlp_stencils(int n, const float *axes, const float *quat, const float *dir, const float *delta,
                      const int32_t *invert, int sub, float noise, uint64_t noise_seed, void *X, float *target,
                      void *stream);

@@ -199,7 +199,8 @@ __global__ void __launch_bounds__(128) k_mlp_targets(int n, const float *axes, c
 //            (a quarter stays open), queued so that the 32 lanes always sample
 //            32 open columns
 //   noise    on the partially filled cells, packed onto the lanes (FP64)
-// and the canonical BF16 row leaves in one 8-byte store per lane.  One block of
+// and the canonical BF16 row leaves in one 8-byte store per lane (in 2-byte stores
+// where X does not lie on an 8-byte boundary; rows are 256 bytes).  One block of
 // 125 sampling threads per stencil, one of which also bisected for the target
 // in FP64, took 16 ms for 65536 stencils at sub = 8; this takes 1.55 ms and the
 // targets 0.08.
@@ -211,7 +212,7 @@ struct StWarp {
     int cnt[128];
     int queue[64];
     uint8_t open[128];
-    __nv_bfloat16 row[128];
+    alignas(16) __nv_bfloat16 row[128];
 };
 
 __global__ void __launch_bounds__(32 * ST_WARPS) k_mlp_stencils(int n, int per, const float *axes, const float *quat,
@@ -225,6 +226,7 @@ __global__ void __launch_bounds__(32 * ST_WARPS) k_mlp_stencils(int n, int per, 
     const long long groups = ((long long)n + per - 1) / per, nw = (long long)gridDim.x * ST_WARPS;
     const int S2 = sub * sub, tot = S2 * sub;
     const int magic = (65536 + sub - 1) / sub;  // c / sub = (c magic) >> 16 for c < 1024, sub <= 32
+    const bool wide = (reinterpret_cast<uintptr_t>(X) & 7) == 0;
     const float h = 1.0f / sub, half = 0.5f * (float)(sub - 1) * h + 1e-6f;  // half a column of samples
     for (long long g = (long long)blockIdx.x * ST_WARPS + (threadIdx.x >> 5); g < groups; g += nw) {
         const int m = (int)min((long long)per, n - g * per);
@@ -362,7 +364,12 @@ __global__ void __launch_bounds__(32 * ST_WARPS) k_mlp_stencils(int n, int per, 
                 s.row[e < 125 ? canon_index(cs, e) : e] = __float2bfloat16_rn(e < 125 ? 2.0f * s.st[e] - 1.0f : 0.f);
             }
             __syncwarp();
-            reinterpret_cast<uint2 *>(X + k * MK)[lane] = reinterpret_cast<const uint2 *>(s.row)[lane];
+            if (wide) {
+                reinterpret_cast<uint2 *>(X + k * MK)[lane] = reinterpret_cast<const uint2 *>(s.row)[lane];
+            } else {
+#pragma unroll
+                for (int t = 0; t < 4; ++t) X[k * MK + lane + 32 * t] = s.row[lane + 32 * t];
+            }
             __syncwarp();
         }
     }
@@ -409,6 +416,7 @@ int fsl_mlp_stencils(int n, const float *axes, const float *quat, const float *d
     if (n < 0 || !axes || !quat || !dir || !delta || !invert || !X || !target || sub < 1 || sub > 32 || noise < 0.f)
         return FSL_EINVAL;
     if (n == 0) return FSL_OK;
+    if (reinterpret_cast<uintptr_t>(X) % sizeof(__nv_bfloat16)) return FSL_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
     const int wide = 152 * 16 * ST_WARPS;  // warps of a full GPU
     // a few stencils per warp fill the lanes of the FP64 set-up; fewer where that would leave SMs idle
