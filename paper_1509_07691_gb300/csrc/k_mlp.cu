@@ -207,7 +207,7 @@ __global__ void __launch_bounds__(128) k_mlp_targets(int n, const float *axes, c
 constexpr int ST_WARPS = 4;
 
 struct StWarp {
-    float frame[32][16];  // R (9), C (3), semi-axes (3), least semi-axis
+    float frame[32][17];  // R (9), C (3), semi-axes (3), bound of |A^-1 R^T|, |R|
     float st[128];
     int cnt[128];
     int queue[64];
@@ -215,7 +215,7 @@ struct StWarp {
     alignas(16) __nv_bfloat16 row[128];
 };
 
-__global__ void __launch_bounds__(32 * ST_WARPS) k_mlp_stencils(int n, int per, const float *axes, const float *quat,
+__global__ void __launch_bounds__(32 * ST_WARPS, 5) k_mlp_stencils(int n, int per, const float *axes, const float *quat,
                                                                 const float *dir, const float *delta,
                                                                 const int *invert, int sub, float noise,
                                                                 unsigned long long noise_seed, __nv_bfloat16 *X) {
@@ -239,7 +239,15 @@ __global__ void __launch_bounds__(32 * ST_WARPS) k_mlp_stencils(int n, int per, 
                 f[9 + r] = (float)c[r];
                 f[12 + r] = (float)a[r];
             }
-            f[15] = fminf(f[12], fminf(f[13], f[14]));
+            // Any quaternion is taken as it is.  R = 1 + 2 w K + 2 K^2 with K the cross product
+            // with (x, y, z), |(x, y, z)|^2 = s2: a normal matrix of eigenvalues 1 and
+            // 1 - 2 s2 +- 2 i w sqrt(s2), whose moduli are 1 for a unit quaternion only
+            // (1.0001 is far above the rounding of e2)
+            const float4 v = make_float4(quat[4 * (g * per + lane)], quat[4 * (g * per + lane) + 1],
+                                         quat[4 * (g * per + lane) + 2], quat[4 * (g * per + lane) + 3]);
+            const float s2 = v.y * v.y + v.z * v.z + v.w * v.w, e = 1.0f - 2.0f * s2;
+            f[16] = 1.0001f * sqrtf(fmaxf(1.0f, e * e + 4.0f * v.x * v.x * s2));
+            f[15] = f[16] / fminf(fabsf(f[12]), fminf(fabsf(f[13]), fabsf(f[14])));
         }
         __syncwarp();
         for (int q = 0; q < m; ++q) {
@@ -250,10 +258,10 @@ __global__ void __launch_bounds__(32 * ST_WARPS) k_mlp_stencils(int n, int per, 
             for (int e = 0; e < 9; ++e) Rm[e] = f[e];
 #pragma unroll
             for (int r = 0; r < 3; ++r) C[r] = f[9 + r];
-            const float inv_a0 = 1.0f / f[12], inv_a1 = 1.0f / f[13], inv_a2 = 1.0f / f[14], lip = 1.0f / f[15];
+            const float inv_a0 = 1.0f / f[12], inv_a1 = 1.0f / f[13], inv_a2 = 1.0f / f[14], lip = f[15];
             // r = |A^-1 R^T (p - C)| is a norm of p - C: over a displacement v its change is
             // at most |grad r . v| + (lip |v|)^2 / (2 (r - lip |v|)), and at most lip |v|.
-            // reach = |v|, gz = bound of |grad r . v| / |v|.  1: all within the reach
+            // reach = |v|, gr = bound of |grad r . v| / |v|.  1: all within the reach
             // inside, 0: none, -1: open.  tol is far above the rounding of the sample test.
             const float tol = 4e-6f * ((fabsf(C[0]) + fabsf(C[1]) + fabsf(C[2]) + 8.0f) * lip + 1.0f);
             auto decide = [&](float px, float py, float pz, float reach, bool along_z) {
@@ -263,7 +271,7 @@ __global__ void __launch_bounds__(32 * ST_WARPS) k_mlp_stencils(int n, int per, 
                 const float r2 = fmaxf(y0 * y0 + y1 * y1 + y2 * y2, 1e-30f), ir = rsqrtf(r2), r = r2 * ir;
                 const float v0 = y0 * inv_a0, v1 = y1 * inv_a1, v2 = y2 * inv_a2;
                 const float gr = along_z ? fabsf(Rm[6] * v0 + Rm[7] * v1 + Rm[8] * v2) * ir
-                                         : sqrtf(v0 * v0 + v1 * v1 + v2 * v2) * ir;
+                                         : f[16] * sqrtf(v0 * v0 + v1 * v1 + v2 * v2) * ir;
                 const float lr = lip * reach, rest = r - lr;
                 float b = lr;
                 if (rest > 0.1f) b = fminf(b, 1.0001f * gr * reach + __fdividef(0.5001f * lr * lr, rest));
