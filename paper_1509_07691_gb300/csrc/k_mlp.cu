@@ -215,20 +215,29 @@ struct StWarp {
     alignas(16) __nv_bfloat16 row[128];
 };
 
+// W warps per stencil: 1, or the ST_WARPS of a block, which share the columns of
+// a stencil (each with a queue of its own) and leave the rest to the first warp.
+template <int W>
 __global__ void __launch_bounds__(32 * ST_WARPS, 5) k_mlp_stencils(int n, int per, const float *axes, const float *quat,
                                                                 const float *dir, const float *delta,
                                                                 const int *invert, int sub, float noise,
                                                                 unsigned long long noise_seed, __nv_bfloat16 *X) {
     __shared__ StWarp smem[ST_WARPS];
-    StWarp &s = smem[threadIdx.x >> 5];
-    const int lane = threadIdx.x & 31;
+    static_assert(W == 1 || W == ST_WARPS, "a warp or a block per stencil");
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, part = W == 1 ? 0 : warp;
+    StWarp &s = smem[W == 1 ? warp : 0];
+    int *queue = smem[warp].queue;
     const unsigned full = 0xffffffffu;
-    const long long groups = ((long long)n + per - 1) / per, nw = (long long)gridDim.x * ST_WARPS;
+    auto sync = [] {
+        if (W == 1) __syncwarp();
+        else __syncthreads();
+    };
+    const long long groups = ((long long)n + per - 1) / per, nw = (long long)gridDim.x * (ST_WARPS / W);
     const int S2 = sub * sub, tot = S2 * sub;
     const int magic = (65536 + sub - 1) / sub;  // c / sub = (c magic) >> 16 for c < 1024, sub <= 32
     const bool wide = (reinterpret_cast<uintptr_t>(X) & 7) == 0;
     const float h = 1.0f / sub, half = 0.5f * (float)(sub - 1) * h + 1e-6f;  // half a column of samples
-    for (long long g = (long long)blockIdx.x * ST_WARPS + (threadIdx.x >> 5); g < groups; g += nw) {
+    for (long long g = W == 1 ? (long long)blockIdx.x * ST_WARPS + warp : blockIdx.x; g < groups; g += nw) {
         const int m = (int)min((long long)per, n - g * per);
         if (lane < m) {
             double R[9], a[3], c[3];
@@ -249,7 +258,7 @@ __global__ void __launch_bounds__(32 * ST_WARPS, 5) k_mlp_stencils(int n, int pe
             f[16] = 1.0001f * sqrtf(fmaxf(1.0f, e * e + 4.0f * v.x * v.x * s2));
             f[15] = f[16] / fminf(fabsf(f[12]), fminf(fabsf(f[13]), fabsf(f[14])));
         }
-        __syncwarp();
+        sync();
         for (int q = 0; q < m; ++q) {
             const long long k = g * per + q;
             const float *f = s.frame[q];
@@ -291,7 +300,7 @@ __global__ void __launch_bounds__(32 * ST_WARPS, 5) k_mlp_stencils(int n, int pe
                 if (v < 0) s.open[nopen + __popc(mk & ((1u << lane) - 1u))] = (uint8_t)e;
                 nopen += __popc(mk);
             }
-            __syncwarp();
+            sync();
             // one column of samples: cell e, column (sx, sy)
             auto column = [&](int item) {
                 const int slot = item >> 10, col = item & 1023;
@@ -310,8 +319,8 @@ __global__ void __launch_bounds__(32 * ST_WARPS, 5) k_mlp_stencils(int n, int pe
                 }
                 if (cnt) atomicAdd(&s.cnt[e], cnt);
             };
-            int queued = 0, slot = 0, col = lane;
-            for (int base = 0; base < nopen * S2; base += 32) {  // warp-uniform
+            int queued = 0, slot = 0, col = lane + 32 * part;
+            for (int base = 32 * part; base < nopen * S2; base += 32 * W) {  // warp-uniform
                 while (col >= S2) {
                     col -= S2;
                     ++slot;
@@ -324,18 +333,22 @@ __global__ void __launch_bounds__(32 * ST_WARPS, 5) k_mlp_stencils(int n, int pe
                     if (v == 1) atomicAdd(&s.cnt[e], sub);
                 }
                 const unsigned mk = __ballot_sync(full, v < 0);
-                if (v < 0) s.queue[queued + __popc(mk & ((1u << lane) - 1u))] = (slot << 10) | col;
+                if (v < 0) queue[queued + __popc(mk & ((1u << lane) - 1u))] = (slot << 10) | col;
                 queued += __popc(mk);
                 __syncwarp();
                 if (queued >= 32) {
                     queued -= 32;
-                    column(s.queue[queued + lane]);
+                    column(queue[queued + lane]);
                     __syncwarp();
                 }
-                col += 32;
+                col += 32 * W;
             }
-            if (lane < queued) column(s.queue[lane]);
-            __syncwarp();
+            if (lane < queued) column(queue[lane]);
+            sync();
+            if (part) {
+                sync();  // the first warp is done with the stencil
+                continue;
+            }
             // fill levels; the partially filled cells (all among the open ones) take the noise
             const bool inv = invert[k] != 0;
 #pragma unroll
@@ -348,10 +361,10 @@ __global__ void __launch_bounds__(32 * ST_WARPS, 5) k_mlp_stencils(int n, int pe
                 int np = 0;
                 for (int b = 0; b < nopen; b += 32) {
                     const int e = b + lane < nopen ? s.open[b + lane] : 0;
-                    const bool part = b + lane < nopen && s.st[e] > 0.f && s.st[e] < 1.f;
-                    const unsigned mk = __ballot_sync(full, part);
+                    const bool cut = b + lane < nopen && s.st[e] > 0.f && s.st[e] < 1.f;
+                    const unsigned mk = __ballot_sync(full, cut);
                     __syncwarp();
-                    if (part) s.open[np + __popc(mk & ((1u << lane) - 1u))] = (uint8_t)e;
+                    if (cut) s.open[np + __popc(mk & ((1u << lane) - 1u))] = (uint8_t)e;
                     np += __popc(mk);
                     __syncwarp();
                 }
@@ -378,7 +391,7 @@ __global__ void __launch_bounds__(32 * ST_WARPS, 5) k_mlp_stencils(int n, int pe
 #pragma unroll
                 for (int t = 0; t < 4; ++t) X[k * MK + lane + 32 * t] = s.row[lane + 32 * t];
             }
-            __syncwarp();
+            sync();
         }
     }
 }
@@ -426,14 +439,20 @@ int fsl_mlp_stencils(int n, const float *axes, const float *quat, const float *d
     if (n == 0) return FSL_OK;
     if (reinterpret_cast<uintptr_t>(X) % sizeof(__nv_bfloat16)) return FSL_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    const int wide = 152 * 16 * ST_WARPS;  // warps of a full GPU
-    // a few stencils per warp fill the lanes of the FP64 set-up; fewer where that would leave SMs idle
-    const int per = std::min(8, std::max(1, n / wide));
+    // A few stencils per warp fill the lanes of the FP64 set-up; fewer where that would
+    // leave SMs idle.  A block per stencil where the stencils fit one round of resident
+    // blocks (5 per SM) and each has columns enough to share: n = 100 at sub = 16 / 32
+    // takes 95 / 306 us with a block each and 255 / 1096 with a warp each (204 / 636 with
+    // one block of 125 sampling threads each), n = 760 at sub = 8 73 against 97; at
+    // sub = 4 760 stencils take 58 either way, at sub = 1 51 against 41, and 2400 at
+    // sub = 8 146 against 120.
+    const int per = std::min(8, std::max(1, n / (152 * 16 * ST_WARPS)));
+    const bool block = n <= 152 * 5 && sub >= 8;
     const long long groups = ((long long)n + per - 1) / per;
-    const int grid = (int)std::min<long long>((groups + ST_WARPS - 1) / ST_WARPS, 152 * 64);
+    const int grid = block ? n : (int)std::min<long long>((groups + ST_WARPS - 1) / ST_WARPS, 152 * 64);
     k_mlp_targets<<<std::min((n + 127) / 128, 152 * 16), 128, 0, s>>>(n, axes, quat, dir, delta, invert, target);
-    k_mlp_stencils<<<grid, 32 * ST_WARPS, 0, s>>>(n, per, axes, quat, dir, delta, invert, sub, noise, noise_seed,
-                                                 static_cast<__nv_bfloat16 *>(X));
+    (block ? k_mlp_stencils<ST_WARPS> : k_mlp_stencils<1>)<<<grid, 32 * ST_WARPS, 0, s>>>(
+        n, per, axes, quat, dir, delta, invert, sub, noise, noise_seed, static_cast<__nv_bfloat16 *>(X));
     return cudaGetLastError() == cudaSuccess ? FSL_OK : FSL_ECUDA;
 }
 
