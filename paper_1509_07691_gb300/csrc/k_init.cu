@@ -134,6 +134,29 @@ __device__ __forceinline__ float level(const Level &g, int x, int y, int z, floa
     return G * g.sign;
 }
 
+// Negative radii: inside() squares the radius of kinds 0, 2 and 3, so that the
+// sign shows at whole cells only.  A cell whose centre is more than one cell
+// outside the sphere of that radius is outside, one more than a cell inside is
+// inside, and the rest is sampled: -1 outside, 1 inside, 0 sampled.
+__device__ int whole_cell(const fsl_geometry &g, double x, double y, double z) {
+    const double dx = x - g.c[0], dy = y - g.c[1], dz = z - g.c[2];
+    const double ex = x - g.c2[0], ey = y - g.c2[1], ez = z - g.c2[2];
+    const double r = sqrt(dx * dx + dy * dy + dz * dz), q = sqrt(ex * ex + ey * ey + ez * ez), e = fabs(g.eps2);
+    bool in = r + 1.0 < g.R, out = r - 1.0 > g.R;
+    if (g.kind == 1) {
+        in = r + 1.0 < g.R * (1.0 - 0.5 * e);
+        out = r - 1.0 > g.R * (1.0 + e);
+    } else if (g.kind == 2) {
+        in = in && z - 1.0 > g.zw;
+        out = out || z + 1.0 < g.zw;
+    } else if (g.kind == 3) {
+        in = in || q + 1.0 < g.R2;
+        out = out && q - 1.0 > g.R2;
+    }
+    const int w = in ? 1 : (out ? -1 : 0);
+    return g.invert ? -w : w;
+}
+
 // Fill levels: the fraction of the sub^3 sample points of a cell that
 // inside() holds for.  Sampling every cell near the surface in FP64 is bound
 // by the FP64 rate (2 FMA per clock and SM): one thread per cell took 180 ms
@@ -158,6 +181,8 @@ __device__ __noinline__ bool sample_inside(const fsl_geometry &g, int S, int x, 
     return inside(g, px, py, pz);
 }
 
+// NEGATIVE: a radius is negative
+template <bool NEGATIVE>
 __global__ void __launch_bounds__(FILL_BLOCK) k_fill(fsl_geometry g, Level lv, int nx, int ny, int nz, float *phi) {
     __shared__ int todo[FILL_BLOCK];
     __shared__ int ntodo;
@@ -167,7 +192,14 @@ __global__ void __launch_bounds__(FILL_BLOCK) k_fill(fsl_geometry g, Level lv, i
     __syncthreads();
     float T, L;
     if (x < nx) {
-        const float G = level(lv, x, y, z, 0.f, 0.f, 0.f, T, L), B = L * CELL_HD + T;
+        float G, B;
+        if (NEGATIVE) {
+            G = (float)whole_cell(g, x, y, z);
+            B = 0.5f;
+        } else {
+            G = level(lv, x, y, z, 0.f, 0.f, 0.f, T, L);
+            B = L * CELL_HD + T;
+        }
         if (G > B) phi[row + x] = 1.0f;
         else if (G < -B) phi[row + x] = 0.0f;
         else todo[atomicAdd(&ntodo, 1)] = x;
@@ -233,15 +265,16 @@ void launch_fill_geometry(const fsl_params &p, const fsl_geometry &g, float *phi
         ok = (split(g.c2[k], l.ci2[k], l.cf2[k]) || g.kind != 3) && ok;
         l.n[k] = (float)g.n[k];
     }
-    l.R = ok ? (float)g.R : NAN;  // NaN: every sample takes the FP64 test
-    l.R2 = (float)g.R2;
+    const bool negative = (g.kind <= 3 && g.R < 0.0) || (g.kind == 3 && g.R2 < 0.0);
+    l.R = ok ? (float)(g.kind == 1 ? g.R : fabs(g.R)) : NAN;  // NaN: every sample takes the FP64 test
+    l.R2 = (float)fabs(g.R2);
     l.eps2 = (float)g.eps2;
     l.nl = 1.0001f * (float)sqrt(g.n[0] * g.n[0] + g.n[1] * g.n[1] + g.n[2] * g.n[2]);
     l.d = (float)g.d;
     l.h0 = (float)g.h0;
     l.amp = (float)g.amp;
     l.iw = (float)(1.0 / g.wavelength);
-    k_fill<<<grid, FILL_BLOCK, 0, s>>>(g, l, p.nx, p.ny, p.nz, phi);
+    (negative ? k_fill<true> : k_fill<false>)<<<grid, FILL_BLOCK, 0, s>>>(g, l, p.nx, p.ny, p.nz, phi);
 }
 
 // ---- initial types (Sec. II) -----------------------------------------------
