@@ -263,14 +263,20 @@ void launch_fill_geometry(const fsl_params &p, const fsl_geometry &g, float *phi
     for (int k = 0; k < 3; ++k) {
         ok = (split(g.c[k], l.ci[k], l.cf[k]) || g.kind > 3) && ok;
         ok = (split(g.c2[k], l.ci2[k], l.cf2[k]) || g.kind != 3) && ok;
-        l.n[k] = (float)g.n[k];
     }
     const bool negative = (g.kind <= 3 && g.R < 0.0) || (g.kind == 3 && g.R2 < 0.0);
     l.R = ok ? (float)(g.kind == 1 ? g.R : fabs(g.R)) : NAN;  // NaN: every sample takes the FP64 test
     l.R2 = (float)fabs(g.R2);
     l.eps2 = (float)g.eps2;
-    l.nl = 1.0001f * (float)sqrt(g.n[0] * g.n[0] + g.n[1] * g.n[1] + g.n[2] * g.n[2]);
-    l.d = (float)g.d;
+    // A half-space by its normal over the largest component: in FP32 a tiny normal is
+    // subnormal or zero, and T counts roundings relative to the terms.  Where the FP64
+    // products themselves can underflow or overflow, or there is no direction: NaN, and
+    // every sample takes the FP64 test.
+    const double big = fmax(fabs(g.n[0]), fmax(fabs(g.n[1]), fabs(g.n[2])));
+    const double scale = big > 1e-280 && big < 1e280 ? big : NAN;
+    for (int k = 0; k < 3; ++k) l.n[k] = (float)(g.n[k] / scale);
+    l.d = (float)(g.d / scale);
+    l.nl = 1.0001f * sqrtf(l.n[0] * l.n[0] + l.n[1] * l.n[1] + l.n[2] * l.n[2]);
     l.h0 = (float)g.h0;
     l.amp = (float)g.amp;
     l.iw = (float)(1.0 / g.wavelength);

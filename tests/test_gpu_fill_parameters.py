@@ -56,3 +56,12 @@ def test_negative_radii(orc, name, invert, sub):
     w = _whole(kind, invert, **kw)
     want = np.where(w > 0, np.float32(1), np.where(w < 0, np.float32(0), _sampled(orc, kind, sub, invert, **kw)))
     assert np.array_equal(_fill(kind, sub, invert, **kw), want)
+
+
+@pytest.mark.parametrize("sub", [1, 5, 16])
+@pytest.mark.parametrize("invert", [0, 1])
+@pytest.mark.parametrize("scale", [1e-320, 1e-300, 1e-160, 7e-44, 3e-42, 1e-39, 1e-30, 1.0, 1e30, 1e160, 1e300, 0.0])
+def test_half_space_normals_of_any_length(orc, scale, invert, sub):
+    n = tuple(scale * v for v in (0.31, -0.52, 0.73))
+    kw = dict(n=n, d=scale * 7.4)
+    assert np.array_equal(_fill("plane", sub, invert, **kw), _sampled(orc, "plane", sub, invert, **kw))
