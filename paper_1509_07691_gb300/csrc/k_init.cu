@@ -134,10 +134,11 @@ __device__ __forceinline__ float level(const Level &g, int x, int y, int z, floa
     return G * g.sign;
 }
 
-// Negative radii: inside() squares the radius of kinds 0, 2 and 3, so that the
-// sign shows at whole cells only.  A cell whose centre is more than one cell
-// outside the sphere of that radius is outside, one more than a cell inside is
-// inside, and the rest is sampled: -1 outside, 1 inside, 0 sampled.
+// Whole cells in FP64 where the level function does not stand for the samples:
+// negative radii (inside() squares the radius of kinds 0, 2 and 3) and non-finite
+// parameters (a pool of wavelength 0 has no samples inside, and whole cells below
+// its crests).  A cell whose centre is more than one cell inside is inside, one
+// more than a cell outside is outside, and the rest is sampled: 1, -1, 0.
 __device__ int whole_cell(const fsl_geometry &g, double x, double y, double z) {
     const double dx = x - g.c[0], dy = y - g.c[1], dz = z - g.c[2];
     const double ex = x - g.c2[0], ey = y - g.c2[1], ez = z - g.c2[2];
@@ -152,6 +153,9 @@ __device__ int whole_cell(const fsl_geometry &g, double x, double y, double z) {
     } else if (g.kind == 3) {
         in = in || q + 1.0 < g.R2;
         out = out && q - 1.0 > g.R2;
+    } else if (g.kind == 4) {
+        in = z + 1.0 < g.h0 - fabs(g.amp);
+        out = z - 1.0 > g.h0 + fabs(g.amp);
     }
     const int w = in ? 1 : (out ? -1 : 0);
     return g.invert ? -w : w;
@@ -181,8 +185,17 @@ __device__ __noinline__ bool sample_inside(const fsl_geometry &g, int S, int x, 
     return inside(g, px, py, pz);
 }
 
-// NEGATIVE: a radius is negative
-template <bool NEGATIVE>
+// 1 or -1: cell (x, y, z) is inside or outside as a whole; 0: open.  WHOLE: as
+// whole_cell says, not the level function.
+template <bool WHOLE>
+__device__ __forceinline__ int decide_cell(const fsl_geometry &g, const Level &lv, int x, int y, int z) {
+    if (WHOLE) return whole_cell(g, x, y, z);
+    float T, L;
+    const float G = level(lv, x, y, z, 0.f, 0.f, 0.f, T, L), B = L * CELL_HD + T;
+    return G > B ? 1 : (G < -B ? -1 : 0);
+}
+
+template <bool WHOLE>
 __global__ void __launch_bounds__(FILL_BLOCK) k_fill(fsl_geometry g, Level lv, int nx, int ny, int nz, float *phi) {
     __shared__ int todo[FILL_BLOCK];
     __shared__ int ntodo;
@@ -192,16 +205,8 @@ __global__ void __launch_bounds__(FILL_BLOCK) k_fill(fsl_geometry g, Level lv, i
     __syncthreads();
     float T, L;
     if (x < nx) {
-        float G, B;
-        if (NEGATIVE) {
-            G = (float)whole_cell(g, x, y, z);
-            B = 0.5f;
-        } else {
-            G = level(lv, x, y, z, 0.f, 0.f, 0.f, T, L);
-            B = L * CELL_HD + T;
-        }
-        if (G > B) phi[row + x] = 1.0f;
-        else if (G < -B) phi[row + x] = 0.0f;
+        const int w = decide_cell<WHOLE>(g, lv, x, y, z);
+        if (w) phi[row + x] = w > 0 ? 1.0f : 0.0f;
         else todo[atomicAdd(&ntodo, 1)] = x;
     }
     __syncthreads();
@@ -280,7 +285,12 @@ void launch_fill_geometry(const fsl_params &p, const fsl_geometry &g, float *phi
     l.h0 = (float)g.h0;
     l.amp = (float)g.amp;
     l.iw = (float)(1.0 / g.wavelength);
-    (negative ? k_fill<true> : k_fill<false>)<<<grid, FILL_BLOCK, 0, s>>>(g, l, p.nx, p.ny, p.nz, phi);
+    // no bound at any cell: non-finite parameters, half-spaces without a direction
+    const bool blind = g.kind <= 3 ? !isfinite(l.R) || (g.kind == 1 && !isfinite(l.eps2)) || (g.kind == 3 && !isfinite(l.R2))
+                       : g.kind == 4 ? !isfinite(l.h0) || !isfinite(l.amp) || !isfinite(l.iw)
+                                     : !isfinite(l.nl) || !isfinite(l.d);
+    const bool whole = negative || (blind && g.kind != 5);
+    (whole ? k_fill<true> : k_fill<false>)<<<grid, FILL_BLOCK, 0, s>>>(g, l, p.nx, p.ny, p.nz, phi);
 }
 
 // ---- initial types (Sec. II) -----------------------------------------------

@@ -65,3 +65,11 @@ def test_half_space_normals_of_any_length(orc, scale, invert, sub):
     n = tuple(scale * v for v in (0.31, -0.52, 0.73))
     kw = dict(n=n, d=scale * 7.4)
     assert np.array_equal(_fill("plane", sub, invert, **kw), _sampled(orc, "plane", sub, invert, **kw))
+
+
+@pytest.mark.parametrize("sub", [1, 4])
+def test_pool_without_a_wavelength(sub):
+    """No sample is inside (the phase is no number), whole cells below the crests are."""
+    z = np.broadcast_to(np.arange(SHAPE[0], dtype=np.float64)[:, None, None], SHAPE)
+    want = (z + 1 < 13.6 - 2.0).astype(np.float32)
+    assert np.array_equal(_fill("pool", sub, 0, h0=13.6, amp=2.0, wavelength=0.0), want)
