@@ -67,9 +67,49 @@ def test_half_space_normals_of_any_length(orc, scale, invert, sub):
     assert np.array_equal(_fill("plane", sub, invert, **kw), _sampled(orc, "plane", sub, invert, **kw))
 
 
+SHAPES = {
+    "sphere": dict(c=C, R=7.3), "mode2": dict(c=C, R=5.5, eps2=0.3), "cap": dict(c=C, R=8.1, zw=14.0),
+    "two_spheres": dict(c=C, R=4.4, c2=C2, R2=5.2), "pool": dict(h0=13.6, amp=3.0, wavelength=1.7),
+    "plane": dict(n=(0.31, -0.52, 0.73), d=7.4),
+}
+
+
+@pytest.mark.parametrize("invert", [0, 1])
+@pytest.mark.parametrize("sub", [1, 2, 3])
+@pytest.mark.parametrize("kind", sorted(SHAPES))
+def test_few_samples(orc, kind, sub, invert):
+    """A thread per cell up to 2^3 samples, a warp per open cell from 3^3 on."""
+    assert np.array_equal(_fill(kind, sub, invert, **SHAPES[kind]), _sampled(orc, kind, sub, invert, **SHAPES[kind]))
+
+
 @pytest.mark.parametrize("sub", [1, 4])
 def test_pool_without_a_wavelength(sub):
     """No sample is inside (the phase is no number), whole cells below the crests are."""
     z = np.broadcast_to(np.arange(SHAPE[0], dtype=np.float64)[:, None, None], SHAPE)
     want = (z + 1 < 13.6 - 2.0).astype(np.float32)
     assert np.array_equal(_fill("pool", sub, 0, h0=13.6, amp=2.0, wavelength=0.0), want)
+
+
+def test_one_sample_costs_less_than_many():
+    """Cells of one sample are not taken by a warp each: 0.3 of the time of 6^3 samples
+    on a pool of short waves, with a warp per cell 0.9 (256 x 256 x 24)."""
+    import torch
+    from paper_1509_07691_gb300 import fsl as F
+    shape = (24, 256, 256)
+    phi = torch.empty(shape, device="cuda")
+
+    def ms(sub):
+        g, P = F.make_geometry("pool", h0=12.3, amp=6.0, wavelength=1.7, sub=sub), F.make_params(shape)
+        v = []
+        for _ in range(6):
+            e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            e[0].record()
+            for _ in range(5):
+                F.fill_geometry(P, g, phi)
+            e[1].record()
+            torch.cuda.synchronize()
+            v.append(e[0].elapsed_time(e[1]))
+        return min(v)
+
+    a, b = ms(1), ms(6)
+    assert a < 0.6 * b, (a, b)
