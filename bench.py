@@ -1004,7 +1004,8 @@ def run_fsl(args):
     flush = torch.empty(L2_FLUSH_BYTES // 4, dtype=torch.float32, device="cuda")
 
     sim.step(args.develop)
-    sim.step(args.warmup)
+    for _ in range(args.warmup):  # by the call that is timed
+        sim.step(1)
     torch.cuda.synchronize()
     st = sim.stats()
     n_fluid, n_if, N = int(st[0] + st[1]), int(st[1]), sim.N

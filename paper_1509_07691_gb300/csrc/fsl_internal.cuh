@@ -114,6 +114,14 @@ __host__ __device__ __forceinline__ int div_by(int n, const FastDiv &f) {
     return (int)(((unsigned long long)(unsigned)n * f.m) >> f.shift);
 }
 
+// The recorded graph that the next of `left` steps from this parity take: 0, 1 one
+// step from parity 0, 1; 2, 3 two steps.  An odd count from parity 1 takes its
+// single step first, so that its pairs start from parity 0 like those of the odd
+// count before it: a caller that steps by one count has every graph after one call.
+inline int next_graph(int left, int parity) {
+    return left >= 2 && !(parity && (left & 1)) ? 2 + parity : parity;
+}
+
 // kernel argument block (passed by value)
 struct Dev {
     int nx, ny, nz;
