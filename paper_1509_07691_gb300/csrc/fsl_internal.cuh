@@ -64,10 +64,18 @@ __device__ __forceinline__ void set_status(int *status, int code) { atomicCAS(st
 
 // Programmatic dependent launch along the serial chain of a step.  A kernel
 // started with launch_pdl may be dispatched while its predecessor on the
-// stream is still running: it calls pdl_wait() before anything else (the wait
-// returns once the predecessor grid has completed and its writes are
-// visible), then pdl_trigger() so that its own successor can be dispatched
-// early in turn.  Both are no-ops in a kernel launched the ordinary way.
+// stream is still running; pdl_wait() returns once the predecessor grid has
+// completed and its writes are visible.  Before the wait a kernel reads only
+// memory that no kernel still running on the stream can write (constants, the
+// network's packed weights in a step, the rows of an epoch), and writes none.
+// pdl_trigger() lets the successor be dispatched early in turn; it comes after
+// the wait, so that completion is transitive.  pdl_enter() does both, for the
+// short list kernels.  A kernel of long or unequal blocks (the network, the
+// triangle fan, the finite differences) does not trigger: its successor's blocks
+// would fill the SMs that empty first, and the list work of the whole step would
+// sit on those (ten steps of a 48^3 droplet with the learned curvature 780 us
+// with the trigger, 668 without; with the triangle fan 509 and 484).
+// All are no-ops in a kernel launched the ordinary way.
 #ifndef FSL_PDL
 #define FSL_PDL 1
 #endif

@@ -148,7 +148,7 @@ constexpr float TR_TWO_PI = 6.28318530717958647692f;
 constexpr float TR_PI = 3.14159265358979323846f;
 
 __global__ void __launch_bounds__(LIST_THREADS) k_tr(Dev d, float *kappa_out) {
-    pdl_enter();
+    pdl_wait();  // and no early trigger: see launch_pdl
     int cnt[1];
     block_counts<1>(d.counts, {d.cif}, cnt);
     const int n = cnt[0];
@@ -349,10 +349,10 @@ __global__ void __launch_bounds__(32 * FD_WARPS) k_fd_warp(const __grid_constant
     __shared__ float s_sm[FD_WARPS][125];
     __shared__ float s_n[FD_WARPS][6][3];
     __shared__ FdTable tab;
-    pdl_enter();
-    if (!WALLS)
+    if (!WALLS)  // constants, staged while the normals still run
         for (int e = threadIdx.x; e < (int)(sizeof(FdTable) / 2); e += blockDim.x)
             reinterpret_cast<uint16_t *>(&tab)[e] = reinterpret_cast<const uint16_t *>(&FD_TABLE)[e];
+    pdl_wait();  // and no early trigger: see launch_pdl
     int cnt[1];
     block_counts<1>(d.counts, {d.cif}, cnt);  // synchronises the block
     const int n = cnt[0];

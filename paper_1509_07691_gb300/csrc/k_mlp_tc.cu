@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(CV_THREADS, 1) k_mlp_curv_tc(Dev d, float *kap
     tc_fence_after();
     // the weights and the tensor memory are in place while the fit before this
     // kernel still runs
-    pdl_enter();
+    pdl_wait();  // and no early trigger: see launch_pdl
     int cnt[1];
     block_counts<1>(d.counts, {d.cif}, cnt);
     const int n = cnt[0];
