@@ -446,7 +446,12 @@ void launch_lsqr(const Dev &d, float *kappa_out, cudaStream_t s) {
 void launch_fd(const Dev &d, float *kappa_out, bool first, cudaStream_t s) {
     static const int g = list_blocks((const void *)k_fd_warp<true>, 32 * FD_WARPS, 16);
     static const int g0 = list_blocks((const void *)k_fd_warp<false>, 32 * FD_WARPS, 16);
-    if (!d.inline_general) launch_pdl(k_fd_warp<true>, g, 32 * FD_WARPS, s, d, kappa_out, 0);
+    // with walls an ordinary launch: the cells whose stencil reaches a wall (1000 times
+    // the work of the others, by one lane) are neighbours in the list, and blocks that
+    // start while the normals drain gather on the SMs that drain first (a step of the
+    // cap of R = 10 in 32^3 1245 us early, 1164 ordinary; a pool whose surface is off the
+    // walls pays 2 of 96 us a step in 128^3)
+    if (!d.inline_general) k_fd_warp<true><<<g, 32 * FD_WARPS, 0, s>>>(d, kappa_out, 0);
     else if (first) k_fd_warp<false><<<g0, 32 * FD_WARPS, 0, s>>>(d, kappa_out, 1);
     else launch_pdl(k_fd_warp<false>, g0, 32 * FD_WARPS, s, d, kappa_out, 0);
 }
