@@ -60,7 +60,8 @@ __global__ void __launch_bounds__(LIST_BLOCK) k_sc_iface(Dev d) {
 // rho and new PDFs, none of which a fit of another cell reads.
 constexpr int IFACE_MIN_BLOCKS = 3;
 
-template <int S, int COLL, int L>
+// OWN: a step (types not frozen) of a domain without obstacles
+template <int S, int COLL, int L, bool OWN>
 __global__ void __launch_bounds__(LIST_BLOCK, IFACE_MIN_BLOCKS) k_curv_iface_fast(const __grid_constant__ Dev d) {
     pdl_enter();
     int cnt[1];
@@ -71,7 +72,8 @@ __global__ void __launch_bounds__(LIST_BLOCK, IFACE_MIN_BLOCKS) k_curv_iface_fas
     const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), nwarps = (int)((gridDim.x * blockDim.x) >> 5);
     int later = 0;  // this warp's deferred cells (steps without obstacles)
     for (int base = gw * CPW; base < n; base += nwarps * CPW)
-        curv_iface_task<S, COLL, L>(d, base, n, lane, gw, nwarps * CPW, later);
+        curv_iface_task<S, COLL, L, OWN>(d, base, n, lane, gw, nwarps * CPW, later);
+    if (!OWN) return;
     __syncwarp();
     for (int j = lane; j < later; j += 32) general_cell_grid<S, COLL>(d, d.slow[own_place(gw, CPW, nwarps * CPW, j)]);
 }
@@ -237,11 +239,15 @@ void launch_iface(const Dev &d, cudaStream_t s) {
 
 template <int S, int COLL>
 void launch_ci(const Dev &d, cudaStream_t s) {
-    static const int gf = list_blocks((const void *)k_curv_iface_fast<S, COLL, FSL_IFACE_LANES>, LIST_BLOCK, 4);
+    static const int go = list_blocks((const void *)k_curv_iface_fast<S, COLL, FSL_IFACE_LANES, true>, LIST_BLOCK, 4);
+    static const int gf = list_blocks((const void *)k_curv_iface_fast<S, COLL, FSL_IFACE_LANES, false>, LIST_BLOCK, 4);
     static const int gs = list_blocks((const void *)k_curv_iface_slow<S, COLL, true>, LIST_BLOCK, 4);
     static const int gz = list_blocks((const void *)k_curv_iface_slow<S, COLL, false>, LIST_BLOCK, 4);
-    launch_pdl(k_curv_iface_fast<S, COLL, FSL_IFACE_LANES>, gf, LIST_BLOCK, s, d);
-    if (d.inline_general && !d.frozen) return;  // the fused kernel finished its deferred fits itself
+    if (d.inline_general && !d.frozen) {  // the fused kernel finishes its deferred fits itself
+        launch_pdl(k_curv_iface_fast<S, COLL, FSL_IFACE_LANES, true>, go, LIST_BLOCK, s, d);
+        return;
+    }
+    launch_pdl(k_curv_iface_fast<S, COLL, FSL_IFACE_LANES, false>, gf, LIST_BLOCK, s, d);
     if (d.frozen) launch_pdl(k_curv_iface_slow<S, COLL, false>, gz, LIST_BLOCK, s, d);
     else launch_pdl(k_curv_iface_slow<S, COLL, true>, gs, LIST_BLOCK, s, d);
 }

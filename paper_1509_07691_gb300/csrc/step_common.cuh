@@ -243,11 +243,11 @@ __device__ __forceinline__ int own_place(int gw, int cells, int stride, int j) {
 
 // LSQR fit and interface stream-collide of the list cells base .. base + 32/L - 1
 // by one warp, L lanes per cell (see k_curv_iface_fast).  A cell whose fit needs
-// the general path is left to k_curv_iface_slow (list d.slow), in a step without
-// obstacles to this warp itself: its later-th such cell is noted in d.slow at the
-// place of the later-th list cell the warp has visited (see own_place), so that no
-// other warp or counter is involved.  The whole warp must call it.
-template <int S, int COLL, int L>
+// the general path is left to k_curv_iface_slow (list d.slow), with OWN to this
+// warp itself: its later-th such cell is noted in d.slow at the place of the
+// later-th list cell the warp has visited (see own_place), so that no other warp
+// or counter is involved.  The whole warp must call it.
+template <int S, int COLL, int L, bool OWN>
 __device__ __forceinline__ void curv_iface_task(const Dev &d, int base, int n, int lane, int gw, int stride, int &later) {
     using St = Store<S>;
     const long long N = d.N;
@@ -438,7 +438,7 @@ __device__ __forceinline__ void curv_iface_task(const Dev &d, int base, int n, i
         }
     }
     if (act && r == L - 1) St::st(d.fdst, i, 0, fo0 + d.omega_e * ((1.0f / 3.0f) * rg * (1.0f - vv) - fo0), d);
-    if (d.inline_general && !d.frozen) {
+    if (OWN) {
         const unsigned dm = __ballot_sync(0xffffffffu, defer && r == 0);
         if (defer && r == 0) d.slow[own_place(gw, 32 / L, stride, later + __popc(dm & ((1u << lane) - 1u)))] = i;
         later += __popc(dm);
