@@ -401,7 +401,7 @@ __global__ void __launch_bounds__(256) k_init_pdfs(Dev d, void *f2) {
     using T = typename Store<S>::T;
     constexpr int V = 16 / sizeof(T);
     const int q = blockIdx.y;
-    T w[V];
+    alignas(16) T w[V];  // read as one 16-byte word
 #pragma unroll
     for (int e = 0; e < V; ++e) {
         float v = 0.f;
