@@ -150,8 +150,8 @@ int fsl_fill_geometry(const fsl_params *params, const fsl_geometry *geom, float 
  * fields->f[1] is a copy of fields->f[0].
  * Queued on `stream` (a cudaStream_t, or NULL for the default stream); returns
  * after that stream has drained, having read back whether any cell has an
- * obstacle neighbour (a domain without one runs its rare general-path LSQR
- * fits inside the fused step kernel instead of a kernel of their own). */
+ * obstacle neighbour (the steps of a domain without one run their general-path
+ * LSQR fits in the kernel that found them, not in a kernel of their own). */
 int fsl_init(const fsl_params *params, const fsl_fields *fields, const float *phi0, int phi0_where,
              const uint8_t *obstacle, int obstacle_where, void *stream, struct fsl_ctx **out);
 

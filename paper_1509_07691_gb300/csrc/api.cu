@@ -184,9 +184,9 @@ Dev dev_for(const fsl_ctx *c, int parity) {
     } while (0)
 
 // After the near-obstacle bits were (re)computed: with no cell next to an
-// obstacle no fit has a contact line, and the fused fit + interface kernel
-// finishes the few fits it defers itself (the general-path kernel is not
-// launched).  Recorded graphs of the other kind are dropped.
+// obstacle no fit has a contact line, and each warp of the fused fit + interface
+// kernel finishes the fits it defers (the general-path kernel is not launched).
+// Recorded graphs of the other kind are dropped.
 int read_near(fsl_ctx *c) {
     CK(cudaMemcpyAsync(c->host_count, c->base.counts + C_NEAR, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
@@ -218,9 +218,9 @@ void enqueue_curvature(const Dev &d, int model, float *kappa_out, bool in_step, 
 // One time step from parity p (see fsl_step), recorded as a graph with two
 // branches: the liquid stream-collide does not need the curvature, so it runs
 // beside normals -> LSQR -> interface stream-collide; both join before the
-// conversion.  The counters of the step are zeroed by its first kernel.  The
-// kernels after the first of each branch start with a programmatic-launch
-// wait, so each is dispatched while its predecessor drains.
+// conversion.  The counters of the step are zeroed by its first kernel.  Most
+// kernels of the curvature branch start with a programmatic-launch wait, so each
+// is dispatched while its predecessor drains (see launch_pdl for the exceptions).
 int enqueue_step_graph(const fsl_ctx *c, int parity) {
     const Dev d = dev_for(c, parity);
     cudaStream_t s = c->cap_stream, side = c->cap_side;

@@ -796,13 +796,6 @@ __device__ __forceinline__ float general_fit_warp(const Dev &d, const Acc &acc, 
     return kap;
 }
 
-// Fast path: FP32 normal equations of the full model for an interface cell
-// with no contact-line cell in its neighbourhood.  The 5x5 Gram matrix
-// A^T A and A^T f are accumulated row by row (independent FMAs), then solved
-// by Cholesky in registers.  The fit is rejected (cell left to the general
-// path) when a contact-line cell is present, when there are fewer than five
-// rows, or when the Cholesky pivots estimate cond(A^T A) above fp64_cond.
-// In three parts so that the rows can be split over several lanes:
 // fill level at any cell (periodic wrap); an obstacle cell takes the
 // reflected fill level of Sec. II.A (kept out of line: callers unroll over
 // their stencils and obstacle cells are rare)
@@ -820,6 +813,13 @@ static __device__ __forceinline__ float phi_ext(const Dev &d, int x, int y, int 
     return phi_reflected(d, x, y, z);
 }
 
+// Fast path: FP32 normal equations of the full model for an interface cell
+// with no contact-line cell in its neighbourhood.  The 5x5 Gram matrix
+// A^T A and A^T f are accumulated row by row (independent FMAs), then solved
+// by Cholesky in registers.  The fit is rejected (cell left to the general
+// path) when a contact-line cell is present, when there are fewer than five
+// rows, or when the Cholesky pivots estimate cond(A^T A) above fp64_cond.
+// In three parts so that the rows can be split over several lanes:
 // lsqr_fast_frame, lsqr_fast_row (for each neighbour slot t of the 3x3x3
 // block, t = (dz+1)*9 + (dy+1)*3 + (dx+1), centre 13), lsqr_fast_solve.
 struct FastFrame {

@@ -165,8 +165,8 @@ struct Dev {
     float cos_theta, sin_theta;
     float scale, inv_scale;  // 16-bit offset storage
     float fp64_cond;
-    // 1: no cell has an obstacle neighbour, so no fit has a contact line and
-    // a step's conversion kernel finishes the few fits the fused kernel deferred
+    // 1: no cell has an obstacle neighbour, so no fit has a contact line and the
+    // fused kernel's warps finish the fits they defer (not with frozen types)
     int inline_general;
     double cos_theta_d, sin_theta_d;
     // learned curvature (FSL_CURV_MLP): packed parameters, judge tolerance
@@ -331,29 +331,6 @@ __device__ __forceinline__ void block_counts(const int *counts, const int (&idx)
     for (int k = 0; k < K; ++k) out[k] = sh[k];
 }
 
-// Block-aggregated append: one global atomic per block.  Every thread of the
-// block must call it (block-uniform control flow; blockDim.x <= 1024).
-__device__ __forceinline__ void block_append(int *list, int *count, bool pred, int value) {
-    __shared__ int warp_cnt[32];
-    __shared__ int base;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = (blockDim.x + 31) >> 5;
-    const unsigned m = __ballot_sync(0xffffffffu, pred);
-    if (lane == 0) warp_cnt[warp] = __popc(m);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int total = 0;
-        for (int w = 0; w < nwarp; ++w) {
-            const int c = warp_cnt[w];
-            warp_cnt[w] = total;
-            total += c;
-        }
-        base = total ? atomicAdd(count, total) : 0;
-    }
-    __syncthreads();
-    if (pred) list[base + warp_cnt[warp] + __popc(m & ((1u << lane) - 1u))] = value;
-    __syncthreads();
-}
-
 // Loop of a list kernel with a warp-uniform trip count, so that warp_append can
 // be used inside: calls body(k, valid) for k = base + lane.
 template <typename Body>
@@ -381,7 +358,6 @@ void launch_prescribe(const Dev &d, float rho, float ux, float uy, float uz, cud
 void launch_seg_compact(const Dev &d, cudaStream_t s);
 void launch_stats(const Dev &d, cudaStream_t s);
 void launch_mass(const Dev &d, double *out, cudaStream_t s);
-void launch_stream_collide(const Dev &d, cudaStream_t s);
 void launch_sc_bulk(const Dev &d, cudaStream_t s);
 void launch_sc_iface(const Dev &d, cudaStream_t s);
 // LSQR curvature and interface stream-collide in one pass (after launch_normals)
