@@ -162,14 +162,20 @@ __device__ double nearest_mean_curvature(const double a[3], const double o[3]) {
 }
 
 // rotation (row-major, FP64) and centre of stencil k's ellipsoid, its surface
-// point at `delta` from the middle cell's centre
+// point at `delta` from the middle cell's centre.  Any quaternion is taken as it
+// is: the matrix is 1 + 2 w K + 2 K^2 with K the cross product with (x, y, z),
+// |(x, y, z)|^2 = s2, a normal matrix of eigenvalues 1 and 1 - 2 s2 +- 2 i w sqrt(s2),
+// whose moduli are 1 for a unit quaternion only.  rn: a bound of its norm (1.0001 is
+// far above the FP32 rounding).
 __device__ __forceinline__ void stencil_frame(long long k, const float *axes, const float *quat, const float *dir,
-                                              const float *delta, double R[9], double a[3], double c[3]) {
+                                              const float *delta, double R[9], double a[3], double c[3], float &rn) {
     const double w = quat[4 * k], x = quat[4 * k + 1], y = quat[4 * k + 2], z = quat[4 * k + 3];
     const double M[9] = {1 - 2 * (y * y + z * z), 2 * (x * y - w * z), 2 * (x * z + w * y),
                          2 * (x * y + w * z), 1 - 2 * (x * x + z * z), 2 * (y * z - w * x),
                          2 * (x * z - w * y), 2 * (y * z + w * x), 1 - 2 * (x * x + y * y)};
     for (int e = 0; e < 9; ++e) R[e] = M[e];
+    const float fw = (float)w, s2 = (float)x * (float)x + (float)y * (float)y + (float)z * (float)z, re = 1.0f - 2.0f * s2;
+    rn = 1.0001f * sqrtf(fmaxf(1.0f, re * re + 4.0f * fw * fw * s2));
     for (int r = 0; r < 3; ++r) a[r] = axes[3 * k + r];
     const double d[3] = {dir[3 * k], dir[3 * k + 1], dir[3 * k + 2]};
     const double sc = 1.0 / sqrt((d[0] / a[0]) * (d[0] / a[0]) + (d[1] / a[1]) * (d[1] / a[1]) +
@@ -183,7 +189,8 @@ __global__ void __launch_bounds__(128) k_mlp_targets(int n, const float *axes, c
                                                      const float *delta, const int *invert, float *target) {
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
         double R[9], a[3], c[3], o[3];
-        stencil_frame(k, axes, quat, dir, delta, R, a, c);
+        float rn;
+        stencil_frame(k, axes, quat, dir, delta, R, a, c, rn);
         for (int r = 0; r < 3; ++r) o[r] = -(R[r] * c[0] + R[3 + r] * c[1] + R[6 + r] * c[2]);  // R^T (0 - C)
         const double H = nearest_mean_curvature(a, o);
         target[k] = (float)(invert[k] ? -H : H);
@@ -241,21 +248,15 @@ __global__ void __launch_bounds__(32 * ST_WARPS, 5) k_mlp_stencils(int n, int pe
         const int m = (int)min((long long)per, n - g * per);
         if (lane < m) {
             double R[9], a[3], c[3];
-            stencil_frame(g * per + lane, axes, quat, dir, delta, R, a, c);
+            float rn;
+            stencil_frame(g * per + lane, axes, quat, dir, delta, R, a, c, rn);
             float *f = s.frame[lane];
             for (int e = 0; e < 9; ++e) f[e] = (float)R[e];
             for (int r = 0; r < 3; ++r) {
                 f[9 + r] = (float)c[r];
                 f[12 + r] = (float)a[r];
             }
-            // Any quaternion is taken as it is.  R = 1 + 2 w K + 2 K^2 with K the cross product
-            // with (x, y, z), |(x, y, z)|^2 = s2: a normal matrix of eigenvalues 1 and
-            // 1 - 2 s2 +- 2 i w sqrt(s2), whose moduli are 1 for a unit quaternion only
-            // (1.0001 is far above the rounding of e2)
-            const float4 v = make_float4(quat[4 * (g * per + lane)], quat[4 * (g * per + lane) + 1],
-                                         quat[4 * (g * per + lane) + 2], quat[4 * (g * per + lane) + 3]);
-            const float s2 = v.y * v.y + v.z * v.z + v.w * v.w, e = 1.0f - 2.0f * s2;
-            f[16] = 1.0001f * sqrtf(fmaxf(1.0f, e * e + 4.0f * v.x * v.x * s2));
+            f[16] = rn;
             f[15] = f[16] / fminf(fabsf(f[12]), fminf(fabsf(f[13]), fabsf(f[14])));
         }
         sync();

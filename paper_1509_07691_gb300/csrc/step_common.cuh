@@ -19,10 +19,11 @@ __device__ __forceinline__ void sources(const Dev &d, int x, int y, int z, int s
 
 // Liquid cells of the active segment s, one lane per cell (see k_sc_bulk).  The
 // pass is bound by instruction issue where the cells come from the L2 or take
-// 16 bits (800 warp instructions a segment with 64-bit index arithmetic, 450 now:
-// on the 256^3 pool 272 -> 260 us a pass in FP32, 265 -> 213 us in FP16), so a PDF is addressed by the unsigned 32-bit index of its cell on a
-// base that is the same for the whole grid (of its direction): nine row offsets
-// and three columns give the 19 sources.
+// 16 bits, so a PDF is addressed by the unsigned 32-bit index of its cell on a base
+// that is the same for the whole grid (of its direction): nine row offsets and
+// three columns give the 19 sources.  With 64-bit index arithmetic a segment took
+// 800 warp instructions, now 470 in FP32 and 550 in 16 bits: 272 -> 260 us a pass in
+// FP32 on the 256^3 pool, 265 -> 213 us in FP16 on the 251 x 251 x 256 pool.
 template <int S, int COLL>
 __device__ __forceinline__ void bulk_segment(const Dev &d, int s, int lane) {
     using St = Store<S>;
