@@ -781,9 +781,9 @@ __device__ __forceinline__ T lsqr_warp(const Acc &acc, uint8_t fi, int lane, Fit
 }
 
 // The general fit by a warp, re-solved in FP64 (the same pipeline) where the
-// FP32 factor is ill conditioned: necks of merging droplets have many such cells
-// (four steps of the merging 384^3 coalescence 1150 us with the re-solve by one
-// lane, 940 with it pipelined).
+// FP32 factor is ill conditioned: necks of merging droplets have such cells (four
+// steps of the merged 384^3 coalescence, 155 of them: 1595 us with the re-solve by
+// one lane, 1185 with it pipelined; 695 before the droplets touch).
 template <typename Acc>
 __device__ __forceinline__ float general_fit_warp(const Dev &d, const Acc &acc, uint8_t fi, int lane, FitRows &rows) {
     float cond;
