@@ -201,12 +201,14 @@ int read_near(fsl_ctx *c) {
     return FSL_OK;
 }
 
+// Finite differences need no normals; a step reads them at contact lines and for
+// normal-weighted excess shares.
+bool fd_starts(const Dev &d) { return d.inline_general && !d.excess_rule; }
+
 // enqueue the curvature of the current state into kappa_out
 // (in_step: for the step's own use; fsl_curvature also leaves the normals)
 void enqueue_curvature(const Dev &d, int model, float *kappa_out, bool in_step, cudaStream_t s) {
-    // finite differences need no normals; the step reads them at contact lines
-    // and for normal-weighted excess shares
-    const bool normals = !in_step || model != FSL_CURV_FD || !d.inline_general || d.excess_rule;
+    const bool normals = !(in_step && model == FSL_CURV_FD && fd_starts(d));
     if (normals) launch_normals(d, s);
     if (model == FSL_CURV_LSQR || model == FSL_CURV_MLP) launch_lsqr(d, kappa_out, s);
     else if (model == FSL_CURV_FD) launch_fd(d, kappa_out, !normals, s);
@@ -221,13 +223,20 @@ void enqueue_curvature(const Dev &d, int model, float *kappa_out, bool in_step, 
 // conversion.  The counters of the step are zeroed by its first kernel.  Most
 // kernels of the curvature branch start with a programmatic-launch wait, so each
 // is dispatched while its predecessor drains (see launch_pdl for the exceptions).
-int enqueue_step_graph(const fsl_ctx *c, int parity) {
+// alone: the only step of its graph.  The branch that is recorded first is
+// dispatched first, and the liquid pass's blocks fill the SMs.  That goes first
+// except in a graph of one step that starts with the finite differences, the
+// longest of the first kernels: step(1) of a 61 x 36 x 60 bubble 42 us, 51 behind the
+// liquid pass (46 with a normals kernel ahead of them); with the fit's normals
+// first the 256^3 droplet and pool lose 5 and 7 %, as finite differences lose
+// 4 % in a graph of two steps of a 96^3 bubble.
+int enqueue_step_graph(const fsl_ctx *c, int parity, bool alone) {
     const Dev d = dev_for(c, parity);
     cudaStream_t s = c->cap_stream, side = c->cap_side;
     CK(cudaEventRecord(c->fork, s));
     CK(cudaStreamWaitEvent(side, c->fork, 0));
-    launch_sc_bulk(d, side);
-    CK(cudaEventRecord(c->join, side));
+    const bool late = alone && c->p.curv_model == FSL_CURV_FD && fd_starts(d);
+    if (!late) launch_sc_bulk(d, side);
     if (c->p.curv_model == FSL_CURV_LSQR) {
         launch_normals(d, s);
         launch_curv_iface(d, s);
@@ -235,6 +244,8 @@ int enqueue_step_graph(const fsl_ctx *c, int parity) {
         enqueue_curvature(d, c->p.curv_model, d.kappa, true, s);
         launch_sc_iface(d, s);
     }
+    if (late) launch_sc_bulk(d, side);
+    CK(cudaEventRecord(c->join, side));
     CK(cudaStreamWaitEvent(s, c->join, 0));
     launch_convert(d, s);
     launch_finalize(d, s);
@@ -246,7 +257,7 @@ int record_graph(fsl_ctx *c, int parity, int steps) {
     cudaGraph_t g;
     CK(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
     int rc = FSL_OK;
-    for (int k = 0; k < steps && rc == FSL_OK; ++k) rc = enqueue_step_graph(c, parity ^ k);
+    for (int k = 0; k < steps && rc == FSL_OK; ++k) rc = enqueue_step_graph(c, parity ^ k, steps == 1);
     cudaError_t e = cudaStreamEndCapture(c->cap_stream, &g);
     if (rc != FSL_OK || e != cudaSuccess) return FSL_ECUDA;
     e = cudaGraphInstantiate(&c->graph[2 * (steps - 1) + parity], g, 0);

@@ -357,7 +357,7 @@ __global__ void __launch_bounds__(32 * FD_WARPS) k_fd_warp(const __grid_constant
     block_counts<1>(d.counts, {d.cif}, cnt);  // synchronises the block
     const int n = cnt[0];
     // by the block that is last to get a cell: the bubble's pressure is a chain of
-    // FP64 operations, 5 us ahead of the first block's cells
+    // FP64 operations, 1 us ahead of the first block's cells
     if (prologue && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) step_prologue(d);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), nw = (int)((gridDim.x * blockDim.x) >> 5);
