@@ -91,8 +91,8 @@ def test_pool_without_a_wavelength(sub):
 
 
 def test_one_sample_costs_less_than_many():
-    """Cells of one sample are not taken by a warp each: 0.3 of the time of 6^3 samples
-    on a pool of short waves, with a warp per cell 0.9 (256 x 256 x 24)."""
+    """Cells of one sample are not taken by a warp each: 0.03 of the time of 6^3 samples
+    on a pool of short waves, with a warp per cell 0.7 (256 x 256 x 24)."""
     import torch
     from paper_1509_07691_gb300 import fsl as F
     shape = (24, 256, 256)

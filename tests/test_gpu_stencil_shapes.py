@@ -37,7 +37,7 @@ def test_small_sets_equal_the_same_rows_of_a_large_one(n, sub):
 
 
 def test_a_few_fine_stencils_are_not_left_to_single_warps():
-    """100 stencils at 32^3 samples against 1520, which fill the GPU a warp each: 0.28 of
+    """100 stencils at 32^3 samples against 1520, which fill the GPU a warp each: 0.26 of
     their time with a block per stencil, 0.7 with a warp per stencil."""
     import torch
     from paper_1509_07691_gb300 import fsl as F
